@@ -318,6 +318,13 @@ sos_status sos_filter_sync_status(sos_filter *f);
  *     carry folded (the folding warp), [9]
  *     correction start, [10] group state observed, [11] state operand posted,
  *     [12]/[24] correction observed, [14]/[25] outputs stored.
+ *   runs of the two solvers above at N = 64 and 7 or 8 groups that are taken strip by strip (per
+ *     unit of 8192 samples, strip after strip, warm-up units included): [0] unit + 1, [13] SM id;
+ *     [19]/[20] strip's block started, its barriers ready (first unit), [21] tables loaded, [22] done;
+ *     [16] loads issued; operand warp: [1] samples landed, [2] operand buffer free, [3] operands
+ *     posted; issuer: [17] products started, [18] issued; epilogue (first warp of the unit's
+ *     warpgroup): [4] accumulator (or samples) observed, [5] terminal states read, [7] lane scan
+ *     done, [9] incoming state observed, [10] row states done, [11] recurrences done, [12] stored.
  *   cyclic reduction, cascade carry (per tile): see the kernel's source.
  *   cyclic reduction, per-section carries (per ticket): [0] ticket + 1,
  *     [1] start, [2] after drawing the ticket, [3] after stage-in, [4 + 3s]

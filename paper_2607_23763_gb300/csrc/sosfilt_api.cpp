@@ -44,6 +44,8 @@ namespace {
 constexpr int kNumN = 3;
 constexpr int kSupportedN[kNumN] = {32, 64, 128};
 constexpr long long kDefaultSpinBudget = 2000000000LL;  // ~1 s of SM clock
+// a filter's ticket counters (eager, captured) and the strip kernel's workspace behind them
+constexpr size_t kTicketBytes = 2 * sizeof(unsigned long long) + sosk::kStripTailBytes;
 
 struct Mat {
     double a, b, c, d;  // row-major 2x2
@@ -79,7 +81,7 @@ int ilog2i(int n) {
 struct NTables {
     int N = 0;
     std::vector<sosk::SecCoef> sec;  // [K]
-    float4 *d_lane_pow = nullptr;    // [K][32]
+    float4 *d_lane_pow = nullptr;    // [K][32]; the two below lie in the same allocation
     float4 *d_grp_pow = nullptr;     // [K][kGrpPowStride]: powers of T^C
     float4 *d_cta_pow = nullptr;     // [K][kGrpPowStride]: powers of the block transition T^(kWarps C)
 };
@@ -156,6 +158,11 @@ struct LanePass {
     // tensor-core kernel only (N = 64, W = kTcGroups): its constant operands and final-state table
     float *d_tcimg = nullptr;        // shared-memory image of the MMA B operands (kTcImageBytes)
     float *d_gtail = nullptr;        // [2 kp][64] state responses G, float32
+    // strip kernel (N = 64): G as its operand image and in float32 behind it, owned by the (64, 7) tables,
+    // and the rows of 64 samples after which the pass's state is forgotten (0: too many)
+    float *d_strip = nullptr;
+    std::vector<float> gresp;        // G in float32, [2 kp][64]
+    int warm_rows = 0;
 };
 
 }  // namespace
@@ -190,7 +197,8 @@ struct sos_filter {
     // workspace
     unsigned long long *d_desc = nullptr;
     size_t desc_groups = 0;  // capacity in groups (per section slot)
-    unsigned long long *d_ticket = nullptr;  // [2]: eager launches' counter, captured launches' counter
+    // [2]: eager launches' counter, captured launches' counter; then the strip kernel's workspace
+    unsigned long long *d_ticket = nullptr;
     unsigned long long ticket_base = 0;
     unsigned int epoch = 0;
     int *d_status = nullptr;
@@ -640,6 +648,132 @@ sos_status build_tc(sos_filter *f, LanePass &ps) {
     return SOS_OK;
 }
 
+// Rows of 64 samples after which a state no longer counts in float32: the least h for which every entry of
+// the zero-input transition over h rows, Q^h, rounds to zero in float32 (is below 2^-150) and so does every
+// later one.  A later power is Q^h Q^j, so the entries of Q^h are held below 2^-150 / (S G), G the largest
+// entry met on the way (a cascade's transition may grow before it decays; 16 times it, for the powers not
+// formed).  Found by binary lifting over the powers Q^(2^k); 0 if 2^14 rows are not enough.
+int strip_memory(const DMat &M1) {
+    constexpr int kBits = 14;
+    std::vector<DMat> q{dpow(M1, 64)};
+    for (int k = 1; k < kBits; ++k) q.push_back(dmul(q.back(), q.back()));
+    double G = 1.0;
+    auto largest = [](const DMat &m) {
+        double v = 0.0;
+        for (double e : m.a) v = std::fabs(e) > v ? std::fabs(e) : v;
+        return v;
+    };
+    for (const DMat &m : q) G = largest(m) > G ? largest(m) : G;
+    const double least = std::ldexp(1.0, -150) / (16.0 * M1.n * G);
+    DMat P = deye(M1.n);
+    int h = 0;  // the largest count whose power still counts
+    for (int k = kBits - 1; k >= 0; --k) {
+        DMat T = dmul(P, q[k]);
+        if (largest(T) >= least) {
+            P = std::move(T);
+            h += 1 << k;
+        }
+    }
+    return h + 1 < (1 << kBits) ? h + 1 : 0;
+}
+
+// How much a cascade amplifies float32 rounding: the error (2-norm over 2-norm of the output) of its
+// sections run one after the other in float32, in direct-form-I order with fused multiply-adds, on 4096
+// samples of fixed noise.
+double float32_noise(const sos_filter *f) {
+    const int K = f->K;
+    std::vector<float> c(4 * static_cast<size_t>(K)), h(2 * static_cast<size_t>(K + 1), 0.f);
+    std::vector<double> d(4 * static_cast<size_t>(K)), hd(2 * static_cast<size_t>(K + 1), 0.0);
+    std::vector<double> b0(K, 1.0);
+    for (int k = 0; k < K; ++k) {
+        const double *q = &f->sos[5 * k];
+        const double s = f->norm ? q[0] : 1.0;
+        if (!f->norm) b0[k] = q[0];
+        const double v[4] = {q[1] / s, q[2] / s, -q[3], -q[4]};
+        for (int j = 0; j < 4; ++j) {
+            d[4 * k + j] = v[j];
+            c[4 * k + j] = static_cast<float>(v[j]);
+        }
+    }
+    double err = 0.0, sum = 0.0;
+    uint32_t seed = 12345;
+    for (int i = 0; i < 4096; ++i) {
+        double u = 0.0;  // four uniforms: variance 1/3
+        for (int r = 0; r < 4; ++r) {
+            seed = seed * 1664525u + 1013904223u;
+            u += static_cast<double>(seed >> 8) / 16777216.0 - 0.5;
+        }
+        const float x = static_cast<float>(u);
+        float v = x * static_cast<float>(f->gain);
+        double w = static_cast<double>(x) * f->gain;
+        for (int k = 0; k < K; ++k) {  // h[2k], h[2k + 1]: the last two inputs of section k
+            const float *q = &c[4 * k], *in = &h[2 * k], *out = &h[2 * k + 2];
+            const float F = std::fmaf(q[0], in[0], std::fmaf(q[1], in[1], static_cast<float>(b0[k]) * v));
+            const float y = std::fmaf(q[2], out[0], std::fmaf(q[3], out[1], F));
+            h[2 * k + 1] = h[2 * k];
+            h[2 * k] = v;
+            v = y;
+            const double *qd = &d[4 * k], *ind = &hd[2 * k], *outd = &hd[2 * k + 2];
+            const double z = b0[k] * w + qd[0] * ind[0] + qd[1] * ind[1] + qd[2] * outd[0] + qd[3] * outd[1];
+            hd[2 * k + 1] = hd[2 * k];
+            hd[2 * k] = w;
+            w = z;
+        }
+        h[2 * K + 1] = h[2 * K];
+        h[2 * K] = v;
+        hd[2 * K + 1] = hd[2 * K];
+        hd[2 * K] = w;
+        err += (v - w) * (v - w);
+        sum += w * w;
+    }
+    return sum > 0.0 ? std::sqrt(err / sum) : 1.0;
+}
+
+// Cascades above this keep the lookback kernels, whose outputs their users have: where rounding is amplified
+// this much two float32 evaluations differ visibly (order-16 resonators at radius 0.999: noise 3e-5, 3e-5
+// between the kernels' outputs, each 2.3e-5 from float64), below it by less than 1e-5 of the signal.
+constexpr double kStripNoise = 1e-5;
+
+// The strip kernel's tables of one pass: the pass's state responses G (state s after sample 63 of an
+// impulse at sample j), as float32 and as the operand image of the tensor cores -- two halves of 32
+// samples, 32 rows of 128 bytes each: rows 0..15 the words' TF32 values rounded to nearest, rows 16..31
+// the rounded remainders, 16-byte chunk j of a row at chunk j ^ (row mod 8) -- and the rows after which the
+// pass's state is forgotten.
+sos_status build_strip(sos_filter *f, LanePass &ps) {
+    constexpr int N = 64;
+    const int kp = ps.kp, S = 2 * kp;
+    std::vector<float> buf(sosk::kStripImgFloats + static_cast<size_t>(S) * N, 0.f);
+    std::vector<double> z(S, 0.0);
+    auto put = [&](int r, int j, float v) {
+        const int c = j & 31;
+        buf[(j >> 5) * (sosk::kStripImgFloats / 2) + r * 32 + ((((c >> 2) ^ (r & 7)) << 2) | (c & 3))] = v;
+    };
+    auto tf32 = [](double v) {  // nearest TF32 value (11 significant bits) of a double
+        float x = static_cast<float>(v);
+        uint32_t u;
+        std::memcpy(&u, &x, sizeof u);
+        u = (u + 0x1000u) & 0xffffe000u;
+        std::memcpy(&x, &u, sizeof x);
+        return x;
+    };
+    for (int m = 0; m < N; ++m) {
+        cascade_step(ps.coef, kp, z, m == 0 ? (ps.k0 == 0 ? f->gain : 1.0) : 0.0);
+        const int j = N - 1 - m;  // the impulse's sample
+        for (int s = 0; s < S; ++s) {
+            const float hi = tf32(z[s]);
+            put(s, j, hi);
+            put(16 + s, j, tf32(z[s] - static_cast<double>(hi)));
+            buf[sosk::kStripImgFloats + static_cast<size_t>(s) * N + j] = static_cast<float>(z[s]);
+        }
+    }
+    ps.warm_rows = strip_memory(ps.M1);
+    ps.gresp.assign(buf.begin() + sosk::kStripImgFloats, buf.end());
+    if (cudaMalloc(&ps.d_strip, buf.size() * sizeof(float)) != cudaSuccess) return SOS_ENOMEM;
+    if (cudaMemcpy(ps.d_strip, buf.data(), buf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+        return SOS_ECUDA;
+    return SOS_OK;
+}
+
 int table_index(int N) {
     for (int i = 0; i < kNumN; ++i)
         if (kSupportedN[i] == N) return i;
@@ -957,6 +1091,14 @@ sos_status launch_lane_pass(sos_filter *f, LanePass &ps, const float *x, float *
     p->spin_budget = f->tuning.spin_budget_cycles ? f->tuning.spin_budget_cycles : kDefaultSpinBudget;
     p->aligned = aligned ? 1 : 0;
     p->tab = ps.d_tab;
+    if (N == 64 && (TC || W == sosk::kLaneW)) {
+        p->gimg = ps.d_strip;
+        p->gtail = ps.d_strip ? ps.d_strip + sosk::kStripImgFloats : nullptr;
+        p->gresp = ps.gresp.data();
+        p->warm_rows = ps.warm_rows;
+        p->norm = f->norm ? 1 : 0;
+        p->tail = sc ? sc->tail : reinterpret_cast<unsigned *>(f->d_ticket + 2);
+    }
     p->trace = f->trace;
     p->trace_tiles = f->trace_blocks;
     for (int j = 0; j < K; ++j) p->sec[j] = ps.sec[j];
@@ -1721,25 +1863,31 @@ sos_status sos_filter_create(int n_sections, const double *sos, const float *zi,
     for (int i = 0; i < kNumN && st == SOS_OK; ++i) {
         std::vector<float4> lp, gp, cp;
         build_tables(f, kSupportedN[i], f->tables[i], lp, gp, cp);
-        if (cudaMalloc(&f->tables[i].d_lane_pow, lp.size() * sizeof(float4)) != cudaSuccess ||
-            cudaMalloc(&f->tables[i].d_grp_pow, gp.size() * sizeof(float4)) != cudaSuccess ||
-            cudaMalloc(&f->tables[i].d_cta_pow, cp.size() * sizeof(float4)) != cudaSuccess) {
+        // one allocation and one copy for the three tables (creation is mostly such calls)
+        lp.insert(lp.end(), gp.begin(), gp.end());
+        lp.insert(lp.end(), cp.begin(), cp.end());
+        NTables &t = f->tables[i];
+        if (cudaMalloc(&t.d_lane_pow, lp.size() * sizeof(float4)) != cudaSuccess) {
             st = SOS_ENOMEM;
             break;
         }
-        if (cudaMemcpy(f->tables[i].d_lane_pow, lp.data(), lp.size() * sizeof(float4), cudaMemcpyHostToDevice) !=
-                cudaSuccess ||
-            cudaMemcpy(f->tables[i].d_grp_pow, gp.data(), gp.size() * sizeof(float4), cudaMemcpyHostToDevice) !=
-                cudaSuccess ||
-            cudaMemcpy(f->tables[i].d_cta_pow, cp.data(), cp.size() * sizeof(float4), cudaMemcpyHostToDevice) !=
-                cudaSuccess)
+        t.d_grp_pow = t.d_lane_pow + (lp.size() - gp.size() - cp.size());
+        t.d_cta_pow = t.d_grp_pow + gp.size();
+        if (cudaMemcpy(t.d_lane_pow, lp.data(), lp.size() * sizeof(float4), cudaMemcpyHostToDevice) != cudaSuccess)
             st = SOS_ECUDA;
     }
     for (int i = 0; i < 2 && st == SOS_OK; ++i) st = build_cascade(f, i == 0 ? 32 : 64, f->cas[i]);
     for (int i = 0; i < 4 && st == SOS_OK; ++i)
         st = build_lane(f, i == 0 ? 32 : 64, i == 2 ? sosk::kLaneWide : i == 3 ? sosk::kTcGroups : sosk::kLaneW,
                         f->lane[i]);
-    for (size_t i = 0; i < f->lane[3].size() && st == SOS_OK; ++i) st = build_tc(f, f->lane[3][i]);
+    const bool strips = float32_noise(f) <= kStripNoise;
+    for (size_t i = 0; i < f->lane[3].size() && st == SOS_OK; ++i) {
+        st = build_tc(f, f->lane[3][i]);
+        if (st == SOS_OK && strips) st = build_strip(f, f->lane[1][i]);
+        f->lane[3][i].d_strip = f->lane[1][i].d_strip;
+        f->lane[3][i].warm_rows = f->lane[1][i].warm_rows;
+        f->lane[3][i].gresp = f->lane[1][i].gresp;
+    }
     if (st == SOS_OK) {
         for (int g = 0; g < sosk::kBatchGeoms; ++g) {
             const LanePass &ps = f->lane[g == 0 ? 1 : 0][0];  // (64, kBatchW) and (32, kBatchW)
@@ -1753,13 +1901,13 @@ sos_status sos_filter_create(int n_sections, const double *sos, const float *zi,
         f->bt.geom = static_cast<signed char>(f->tuning.N == sosk::kBatchNs ? 1 : f->tuning.N ? 0 : -1);
     }
     if (st == SOS_OK) {
-        if (cudaMalloc(&f->d_ticket, 2 * sizeof(unsigned long long)) != cudaSuccess ||  // eager, captured
+        if (cudaMalloc(&f->d_ticket, kTicketBytes) != cudaSuccess ||
             cudaMalloc(&f->d_status, sizeof(int)) != cudaSuccess ||
             cudaMalloc(&f->d_state, sizeof(float) * 2 * n_sections) != cudaSuccess)
             st = SOS_ENOMEM;
     }
     if (st == SOS_OK) {
-        if (cudaMemset(f->d_ticket, 0, 2 * sizeof(unsigned long long)) != cudaSuccess ||
+        if (cudaMemset(f->d_ticket, 0, kTicketBytes) != cudaSuccess ||
             cudaMemset(f->d_status, 0, sizeof(int)) != cudaSuccess)
             st = SOS_ECUDA;
         std::vector<float> z(2 * n_sections, 0.f);
@@ -1785,8 +1933,6 @@ sos_status sos_filter_destroy(sos_filter *f) {
     cudaDeviceSynchronize();
     for (auto &t : f->tables) {
         if (t.d_lane_pow) cudaFree(t.d_lane_pow);
-        if (t.d_grp_pow) cudaFree(t.d_grp_pow);
-        if (t.d_cta_pow) cudaFree(t.d_cta_pow);
     }
     for (auto &ct : f->cas)
         for (auto &ps : ct.passes) {
@@ -1800,6 +1946,7 @@ sos_status sos_filter_destroy(sos_filter *f) {
             if (ps.d_Mm) cudaFree(ps.d_Mm);
             if (ps.d_tcimg) cudaFree(ps.d_tcimg);
             if (ps.d_gtail) cudaFree(ps.d_gtail);
+            if (ps.d_strip && &v == &f->lane[1]) cudaFree(ps.d_strip);
         }
     if (f->d_desc) cudaFree(f->d_desc);
     if (f->d_ticket) cudaFree(f->d_ticket);

@@ -135,6 +135,13 @@ size_t cascade_smem(int K, int N);
 constexpr int kLaneW = 7;    // compute warps per block, one group each; a tile is kLaneW groups
 constexpr int kLaneWide = 10;  // the wide variant at N = 64: 10 groups per tile (sos_tuning.groups_per_cta)
 
+// ---- PH kernel over strips (sosfilt_strip.cuh): one strip of consecutive samples per block, for cascades
+// whose memory is finite in float32
+constexpr int kStripUnit = 8192;        // samples of a unit of its work: 128 rows of 64
+constexpr int kStripMax = 256;          // strips of a run (at most one per SM)
+constexpr size_t kStripTailBytes = 128 + 4 * kStripMax;  // a run's workspace, zero between runs
+constexpr int kStripImgFloats = 2048;   // tensor-core image of the state responses (8 KB)
+
 // Per-section constants of the skewed-pass kernel, in the kernel's domain (b / b0 and b0 = 1 when
 // normalized; carried state = zscale * true state).
 struct LaneSec {
@@ -166,6 +173,14 @@ struct LaneParams {
     // blocks (k, j), j < k, of the lane transition M_N, row-major 2x2 at k (k - 1) / 2 + j
     float4 MX[K > 1 ? K * (K - 1) / 2 : 1];
     float A_tail[2 * K * (K + 1)];  // packed cascade transition over m_last + 1 samples
+    // the strip kernel's (kernels at N = 64): state responses as the tensor cores' operand image and in
+    // float32 ([2K][64]), rows of 64 samples until the cascade's state is forgotten in float32 (0: not
+    // within 2^14), workspace (nullptr: none), b0-normalized
+    const float *gimg, *gtail;
+    const float *gresp;  // gtail in host memory
+    int warm_rows;
+    int norm;
+    unsigned *tail;
 };
 
 // Phase trace of the skewed-pass kernel, per tile (global timer, ns): [0] tile + 1; coordinator:
@@ -286,11 +301,25 @@ struct BatchAllParams {
 cudaError_t launch_batch_all(const BatchAllParams &p, long long grid, cudaStream_t s);
 int batch_all_blocks_per_sm();
 
-// Device memory for the lookback descriptors and the ticket counter of one cascade run.
+// Runs a pass by strips where that is the better way (returns true, with the launch's status in err);
+// otherwise false, and nothing was launched.  grid: what the caller's own kernel would use, added with
+// the tile count to the eager launches' ticket counter as that kernel would leave it.
+template <int K>
+bool launch_strip(const LaneParams<K> &p, long long grid, cudaStream_t s, cudaError_t &err);
+#define SOSK_DECLARE_STRIP(K) \
+    template <>               \
+    bool launch_strip<K>(const LaneParams<K> &p, long long grid, cudaStream_t s, cudaError_t &err);
+SOSK_DECLARE_STRIP(1) SOSK_DECLARE_STRIP(2) SOSK_DECLARE_STRIP(3) SOSK_DECLARE_STRIP(4)
+SOSK_DECLARE_STRIP(5) SOSK_DECLARE_STRIP(6) SOSK_DECLARE_STRIP(7) SOSK_DECLARE_STRIP(8)
+#undef SOSK_DECLARE_STRIP
+
+// Device memory for the lookback descriptors and the ticket counter of one cascade run, and the strip
+// kernel's workspace (kStripTailBytes, zero; nullptr: none).
 struct Scratch {
     unsigned long long *desc;
     size_t desc_words;
     unsigned long long *ticket;
+    unsigned *tail;
 };
 
 // Launch one pass.  Returns cudaSuccess or the launch error.

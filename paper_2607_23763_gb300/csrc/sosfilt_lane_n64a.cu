@@ -10,6 +10,8 @@ KernelOnce g_once;
 
 template <int K, bool NORM>
 cudaError_t launch_one(const LaneParams<K> &p, long long grid, cudaStream_t s) {
+    cudaError_t se = cudaSuccess;
+    if (launch_strip<K>(p, grid, s, se)) return se;  // by strips where the cascade's memory allows
     auto kern = sos_lane_kernel<K, 64, NORM, 7>;
     constexpr size_t smem = lane_smem_bytes<K, 64, 7>();
     cudaError_t e = raise_smem_once(g_once<K, NORM>, kern, smem);

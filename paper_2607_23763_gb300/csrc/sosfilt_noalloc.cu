@@ -22,12 +22,14 @@ sos_status run_lane_scratch(sos_filter *f, const float *x, float *y, int64_t n, 
 
 namespace {
 
-// Word 0: ticket counter; words 32..: lookback descriptors (tag << 32 | float bits).  Sized for
+// Word 0: ticket counter; then the strip kernel's workspace (left zero by every run) and the lookback
+// descriptors (tag << 32 | float bits).  Sized for
 // SOS_NOALLOC_MAX_SAMPLES samples per call (PH tiles of 7 x 2048 samples, two slots of up to 16
 // words each).
 constexpr size_t kDescWords =
     (static_cast<size_t>(SOS_NOALLOC_MAX_SAMPLES) / (sosk::kLaneW * sosk::kL * 64) + 1) * 2 * 2 * sosk::kMaxPass;
-constexpr size_t kScratchWords = 32 + kDescWords;
+constexpr size_t kDescAt = 32 + sosk::kStripTailBytes / sizeof(unsigned long long);
+constexpr size_t kScratchWords = kDescAt + kDescWords;
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kScratchWords];
 
@@ -60,7 +62,8 @@ extern "C" sos_status sos_filter_run_noalloc(sos_filter *f, const float *x_dev, 
     }
     sosk::Scratch sc;
     sc.ticket = g_ptr[dev];
-    sc.desc = g_ptr[dev] + 32;
+    sc.tail = reinterpret_cast<unsigned *>(g_ptr[dev] + 32);
+    sc.desc = g_ptr[dev] + kDescAt;
     sc.desc_words = kDescWords;
     return sosk::run_lane_scratch(f, x_dev, y_dev, n, zi_dev, zf_dev, static_cast<cudaStream_t>(stream), sc,
                                   next_epoch_dev);

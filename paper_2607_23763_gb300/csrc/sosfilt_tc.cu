@@ -46,6 +46,8 @@ bool encode_rows(CUtensorMap *tm, const float *base, long long rows) {
 
 template <int K>
 cudaError_t launch_k(const LaneParams<K> &p, const float *img, const float *gtail, long long grid, cudaStream_t s) {
+    cudaError_t se = cudaSuccess;
+    if (launch_strip<K>(p, grid, s, se)) return se;  // by strips where the cascade's memory allows
     TcParams<K> P;
     std::memset(&P, 0, sizeof(P));
     P.p = p;

@@ -39,6 +39,7 @@
 #include <cstring>
 
 #include "sosfilt_lane.cuh"
+#include "sosfilt_tcgen05.cuh"
 
 namespace sosk {
 
@@ -49,7 +50,7 @@ constexpr int kTcW = 4 * kTcUnits;                // groups per tile
 static_assert(kTcW == kTcGroups, "tile geometry");
 constexpr int kTcDS = 6;                          // accumulator slots
 constexpr int kTcCols = 80;                       // accumulator columns: 64 outputs, 16 state words
-constexpr int kTcTmemCols = 512;                  // tensor memory allocated (kTcDS * kTcCols rounded up)
+static_assert(kTcDS * kTcCols <= 512, "tensor memory columns");
 constexpr int kTcThreads = 416;                   // 13 warps
 constexpr int kTcCoord1 = 1;                      // the second coordinator warp
 constexpr int kTcB1 = 2 * kTcCols * 128;          // one B1 image (two K halves of 80 rows x 128 B)
@@ -101,80 +102,6 @@ template <int K>
 constexpr size_t tc_smem_bytes() {
     return 1024 + TcDims<K>::OFF_TAB + sizeof(float) * TcDims<K>::T_END;  // 1024: alignment of the base
 }
-
-// ---- tcgen05, TMA and synchronisation primitives
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ unsigned long long tc_sdesc(unsigned addr) {
-    return static_cast<unsigned long long>((addr & 0x3FFFF) >> 4) | (1ULL << 16) | (64ULL << 32) | (1ULL << 46) |
-           (2ULL << 61);
-}
-
-// Instruction descriptor: D float32, A and B TF32 read K-major, M = 128, N columns.
-__host__ __device__ constexpr unsigned tc_idesc(int n) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<unsigned>(n >> 3) << 17) | (8u << 24);
-}
-
-__device__ __forceinline__ void tc_mma(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc,
-                                       unsigned acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_commit(unsigned long long *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-// 16 consecutive accumulator columns of the warp's 32 lanes: thread t receives lane base + t.
-__device__ __forceinline__ void tc_ld16(unsigned taddr, float (&v)[16]) {
-    unsigned r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void *smem, const CUtensorMap *tm, int x, long long y,
-                                            unsigned long long *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_u32(smem)),
-        "l"(reinterpret_cast<unsigned long long>(tm)), "r"(x), "r"(static_cast<int>(y)), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap *tm, int x, long long y, const void *smem) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                     reinterpret_cast<unsigned long long>(tm)),
-                 "r"(x), "r"(static_cast<int>(y)), "r"(smem_u32(smem))
-                 : "memory");
-}
-
-__device__ __forceinline__ void named_bar_sync(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// Byte offset of float c (0..31) of row r in a 128-byte-swizzled K-major block of rows: 16-byte
-// chunk j of row r sits at chunk j ^ (r mod 8).
-__host__ __device__ constexpr unsigned tc_swz(int r, int c) {
-    return static_cast<unsigned>(r * 128 + ((((c >> 2) ^ (r & 7)) << 4) | ((c & 3) << 2)));
-}
-
-// TF32 remainder of a float32: x minus its upper 19 bits (exact).
-__device__ __forceinline__ float tf32_rem(float x) { return x - __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
 template <int K>
 __global__ void __launch_bounds__(kTcThreads, 1) sos_tc_kernel(const __grid_constant__ TcParams<K> P) {
@@ -250,10 +177,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sos_tc_kernel(const __grid_cons
         }
     }
     if (warp == 2) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(kTcTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_alloc512(&tmem_base);
     }
     fence_proxy_async_smem();  // the operand image is read by the tensor cores
     tc_fence_before();
@@ -642,7 +566,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sos_tc_kernel(const __grid_cons
     __syncthreads();
     if (warp == 2) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
+        tc_dealloc512(tmem);
     }
 }
 

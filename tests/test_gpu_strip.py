@@ -1,0 +1,150 @@
+"""The strip kernel (one strip of the signal per thread block, its incoming state from a warm-up) against
+the float64 oracle at the sizes where it can go wrong, and against the lookback kernel.
+
+Bounds: the suite's stated ones (1e-4 of the peak up to pole radius 0.99, 2e-3 beyond).
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from workloads import designs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+ROW, UNIT, SMS = 64, 8192, 152  # samples of a row and of a unit of 128 rows; strips of a long signal
+
+
+@pytest.fixture(scope="module")
+def dev():
+    from paper_2607_23763_gb300 import build
+    build.build()
+    return torch.device("cuda:0")
+
+
+def _filter(sos, **kw):
+    from paper_2607_23763_gb300 import SosFilter
+    return SosFilter(sos, **kw)
+
+
+# the edges of rows, units, strips of half a unit, strips of one unit and of several, one strip per SM
+SIZES = [1, ROW - 1, ROW, ROW + 1, UNIT - 1, UNIT, UNIT + 1, UNIT + UNIT // 2, 3 * UNIT + ROW, SMS * UNIT // 2 - 1,
+         SMS * UNIT // 2 + 1, SMS * (UNIT - 10 * ROW) + 3, SMS * UNIT + 1, 3 * SMS * UNIT + 77]
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("order,cutoff", [(2, 0.2), (4, 0.3), (6, 0.1), (10, 0.1), (16, 0.05)])
+def test_sizes_alignment_and_state(dev, order, cutoff, n):
+    """Every size with an initial and a final state, aligned, at odd offsets of input and output, in place
+    with the final state over the initial one; all match the oracle, and the in-place result is the
+    out-of-place one bit for bit."""
+    sos = designs.butter_lowpass(order, cutoff)
+    K = order // 2
+    x = workloads.normal_f32(7 + order, n)
+    zi = (0.01 * np.random.default_rng(n).standard_normal((K, 2))).astype(np.float32)
+    ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
+    f = _filter(sos)
+    first = None
+    for ox, oy in [(0, 0), (1, 2), (3, 0), (0, 1)]:
+        xd = torch.empty(n + ox, device=dev)[ox:]
+        xd.copy_(torch.from_numpy(x))
+        y = torch.full((n + oy + 8,), 7.0, device=dev)
+        z, zf = torch.from_numpy(zi).to(dev), torch.empty(K, 2, device=dev)
+        f.run(xd, y[oy:oy + n], zi=z, zf=zf)
+        assert f.sync_status() == 0
+        got = y.cpu().numpy()
+        assert np.all(got[:oy] == 7.0) and np.all(got[oy + n:] == 7.0)  # nothing written outside
+        got = got[oy:oy + n]
+        assert oracle.rel_err(got, ref) < 1e-4
+        assert np.abs(zf.cpu().numpy() - zref).max() < 1e-4 * np.abs(zref).max()
+        if first is None:
+            first = got
+    xd, z = torch.from_numpy(x).to(dev), torch.from_numpy(zi).to(dev)
+    f.run(xd, xd, zi=z, zf=z)
+    assert f.sync_status() == 0
+    assert np.array_equal(xd.cpu().numpy(), first)
+    assert np.abs(z.cpu().numpy() - zref).max() < 1e-4 * np.abs(zref).max()
+    f.close()
+
+
+@pytest.mark.parametrize("order", [2, 8, 16])
+@pytest.mark.parametrize("n", [40000, 1 << 21, (1 << 23) + 5])
+def test_matches_the_lookback_kernel(dev, order, n):
+    """The same signal through the lookback kernel (10 groups per tile, which never takes strips)."""
+    sos = designs.butter_lowpass(order, 0.1)
+    x = torch.randn(n, device=dev, generator=torch.Generator(device=dev).manual_seed(n))
+    a, b = _filter(sos), _filter(sos, tuning={"solver": 2, "groups_per_cta": 10})
+    za, zb = torch.empty(order // 2, 2, device=dev), torch.empty(order // 2, 2, device=dev)
+    ya, yb = a.run(x, zf=za), b.run(x, zf=zb)
+    assert a.sync_status() == 0 and b.sync_status() == 0
+    assert float((ya - yb).abs().max()) < 2e-5 * float(yb.abs().max())
+    assert float((za - zb).abs().max()) < 2e-5 * float(zb.abs().max())
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("radius", [0.9, 0.999, 0.99999])
+def test_long_memory(dev, radius):
+    """Cascades that remember for a part of a strip, for several units, and for longer than a strip (those
+    run the lookback kernel), on a decaying impulse whose tail crosses every strip."""
+    sos = designs.resonator_bank(4, radius=radius)
+    n = 1 << 21
+    x = np.zeros(n, np.float32)
+    x[100] = 1.0
+    x[n // 2:] = workloads.normal_f32(3, n - n // 2)
+    f = _filter(sos)
+    y = f.run(torch.from_numpy(x).to(dev))
+    assert f.sync_status() == 0
+    ref = oracle.sosfilt(sos, x)
+    got = y.cpu().numpy()
+    assert oracle.rel_err(got, ref) < 2e-3
+    assert oracle.rel_err(got[:n // 2], ref[:n // 2]) < 2e-3
+    f.close()
+
+
+@pytest.mark.parametrize("order", [4, 16])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("n,at", [(5000, 4000), (1 << 20, 70001), (1 << 20, (1 << 20) - 2), (3 * SMS * UNIT, 9 * UNIT)])
+def test_a_value_that_is_not_finite_spreads_to_the_end(dev, order, bad, n, at):
+    """What follows a NaN or an infinity in a recurrence is not finite, to the signal's end and in the final
+    state, also in the strips that never saw it; what comes before is untouched.  The next run is clean."""
+    sos = designs.butter_lowpass(order, 0.2)
+    x = workloads.normal_f32(5, n)
+    ref, zref = oracle.sosfilt(sos, x, return_state=True)
+    f = _filter(sos)
+    xd = torch.from_numpy(x).to(dev)
+    xb = xd.clone()
+    xb[at] = bad
+    zf = torch.empty(order // 2, 2, device=dev)
+    y = f.run(xb, zf=zf).cpu().numpy()
+    assert f.sync_status() == 0
+    assert oracle.rel_err(y[:at], ref[:at]) < 1e-4
+    assert not np.isfinite(y[at:]).any()
+    assert not np.isfinite(zf.cpu().numpy()).any()
+    y = f.run(xd, zf=zf).cpu().numpy()
+    assert oracle.rel_err(y, ref) < 1e-4
+    assert np.abs(zf.cpu().numpy() - zref).max() < 1e-4 * np.abs(zref).max()
+    f.close()
+
+
+def test_streams_and_filters_at_once(dev):
+    """Eight filters on eight streams, in place, overlapping on the device: each as if alone."""
+    sos = designs.butter_lowpass(8, 0.1)
+    n = (1 << 20) + 3
+    xs = [torch.randn(n, device=dev) for _ in range(8)]
+    fs = [_filter(sos) for _ in xs]
+    want = [f.run(x) for f, x in zip(fs, xs)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in xs]
+    for _ in range(3):
+        ys = [x.clone() for x in xs]
+        torch.cuda.synchronize()
+        for f, y, s in zip(fs, ys, streams):
+            f.run(y, y, stream=s)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(ys, want))
+    assert all(f.sync_status() == 0 for f in fs)
+    for f in fs:
+        f.close()
