@@ -101,13 +101,14 @@ DMat deye(int n) {
     return r;
 }
 
+// Product of lower block-triangular matrices of 2 x 2 blocks (every transition of a cascade is one).
 DMat dmul(const DMat &x, const DMat &y) {
     DMat r(x.n);
     for (int i = 0; i < x.n; ++i)
-        for (int k = 0; k < x.n; ++k) {
+        for (int k = 0; k <= (i | 1); ++k) {
             const double v = x.at(i, k);
             if (v == 0.0) continue;
-            for (int j = 0; j < x.n; ++j) r.at(i, j) += v * y.at(k, j);
+            for (int j = 0; j <= (k | 1); ++j) r.at(i, j) += v * y.at(k, j);
         }
     return r;
 }
@@ -158,10 +159,13 @@ struct LanePass {
     // tensor-core kernel only (N = 64, W = kTcGroups): its constant operands and final-state table
     float *d_tcimg = nullptr;        // shared-memory image of the MMA B operands (kTcImageBytes)
     float *d_gtail = nullptr;        // [2 kp][64] state responses G, float32
-    // strip kernel (N = 64): G as its operand image and in float32 behind it, owned by the (64, 7) tables,
-    // and the rows of 64 samples after which the pass's state is forgotten (0: too many)
+    // strip kernel (N = 64): whether the tensor cores form its outputs, its operand image (then the
+    // tensor-core kernel's, else G's, owned by the (64, 7) tables), G in float32 on the device and here,
+    // [2 kp][64], and the rows of 64 samples after which the pass's state is forgotten (0: too many)
+    bool products = false;
     float *d_strip = nullptr;
-    std::vector<float> gresp;        // G in float32, [2 kp][64]
+    const float *gimg = nullptr, *gtail = nullptr;
+    std::vector<float> gresp;
     int warm_rows = 0;
 };
 
@@ -586,7 +590,9 @@ sos_status build_lane(sos_filter *f, int N, int W, std::vector<LanePass> &out) {
 // basis H[m][s].  Each value is split into its TF32 head (upper 19 bits of the float32) and the
 // float32 remainder, laid out as the kernel's shared memory holds them: K-major rows of 128 bytes
 // whose 16-byte chunk j sits at chunk j ^ (row mod 8).
-sos_status build_tc(sos_filter *f, LanePass &ps) {
+// `nearest`: the heads rounded to nearest and the remainders to what the tensor core reads of them, so that
+// the split errs by 2^-24 with either sign (for the strip kernel); else both cut.
+sos_status build_tc(sos_filter *f, LanePass &ps, bool nearest) {
     constexpr int N = 64, R1 = 80, HB = 2 * R1 * 128;  // samples per row, B1 rows, bytes of one B1 image
     const int kp = ps.kp, S = 2 * kp;
     const double gain = ps.k0 == 0 ? f->gain : 1.0;
@@ -609,14 +615,15 @@ sos_status build_tc(sos_filter *f, LanePass &ps) {
         const size_t off = base + static_cast<size_t>(r) * 128 + ((((c >> 2) ^ (r & 7)) << 4) | ((c & 3) << 2));
         std::memcpy(&img[off], &v, sizeof v);
     };
-    auto head = [](double v) {
+    auto head = [nearest](double v) {
         float x = static_cast<float>(v);
         uint32_t u;
         std::memcpy(&u, &x, sizeof u);
-        u &= 0xffffe000u;
+        u = (nearest ? u + 0x1000u : u) & 0xffffe000u;
         std::memcpy(&x, &u, sizeof x);
         return x;
     };
+    auto remainder = [&](double v) { return nearest ? head(v) : static_cast<float>(v); };
     for (int n = 0; n < R1; ++n)
         for (int j = 0; j < N; ++j) {
             double v = 0.0;
@@ -624,7 +631,7 @@ sos_status build_tc(sos_filter *f, LanePass &ps) {
                 v = n >= j ? h[n - j] : 0.0;
             else if (n - N < S)
                 v = g[static_cast<size_t>(N - 1 - j) * S + (n - N)];
-            const float hi = head(v), lo = static_cast<float>(v - static_cast<double>(hi));
+            const float hi = head(v), lo = remainder(v - static_cast<double>(hi));
             const size_t half = static_cast<size_t>(j >> 5) * (HB / 2);
             put(half, n, j & 31, hi);
             put(HB + half, n, j & 31, lo);
@@ -632,7 +639,7 @@ sos_status build_tc(sos_filter *f, LanePass &ps) {
     for (int m = 0; m < N; ++m)
         for (int k = 0; k < S; ++k) {
             const double v = H[static_cast<size_t>(k) * N + m];
-            const float hi = head(v), lo = static_cast<float>(v - static_cast<double>(hi));
+            const float hi = head(v), lo = remainder(v - static_cast<double>(hi));
             put(2 * HB, m, k, hi);
             put(2 * HB, m, 16 + k, lo);
         }
@@ -678,7 +685,7 @@ int strip_memory(const DMat &M1) {
 }
 
 // How much a cascade amplifies float32 rounding: the error (2-norm over 2-norm of the output) of its
-// sections run one after the other in float32, in direct-form-I order with fused multiply-adds, on 4096
+// sections run one after the other in float32, in direct-form-I order with fused multiply-adds, on 2048
 // samples of fixed noise.
 double float32_noise(const sos_filter *f) {
     const int K = f->K;
@@ -697,7 +704,7 @@ double float32_noise(const sos_filter *f) {
     }
     double err = 0.0, sum = 0.0;
     uint32_t seed = 12345;
-    for (int i = 0; i < 4096; ++i) {
+    for (int i = 0; i < 2048; ++i) {
         double u = 0.0;  // four uniforms: variance 1/3
         for (int r = 0; r < 4; ++r) {
             seed = seed * 1664525u + 1013904223u;
@@ -733,13 +740,20 @@ double float32_noise(const sos_filter *f) {
 // this much two float32 evaluations differ visibly (order-16 resonators at radius 0.999: noise 3e-5, 3e-5
 // between the kernels' outputs, each 2.3e-5 from float64), below it by less than 1e-5 of the signal.
 constexpr double kStripNoise = 1e-5;
+// Below this noise the default solver's strips take their outputs from the recurrences, from it on from the
+// tensor cores, whose products err by 2e-7 to 3e-7 of the signal whatever the cascade: more than recurrences of
+// this little noise (order 12 at 0.4 Nyquist: 1.7e-7 against 3.1e-7), less than noisier ones (order 16 at
+// 0.2: 3.5e-7 against 3.4e-7; order 8 at 0.1: 1.4e-6 against 3.0e-7).  The tensor-core solver's always come
+// from the products.
+constexpr double kStripProductsNoise = 5e-7;
 
 // The strip kernel's tables of one pass: the pass's state responses G (state s after sample 63 of an
-// impulse at sample j), as float32 and as the operand image of the tensor cores -- two halves of 32
-// samples, 32 rows of 128 bytes each: rows 0..15 the words' TF32 values rounded to nearest, rows 16..31
-// the rounded remainders, 16-byte chunk j of a row at chunk j ^ (row mod 8) -- and the rows after which the
-// pass's state is forgotten.
-sos_status build_strip(sos_filter *f, LanePass &ps) {
+// impulse at sample j) in float32, the rows after which the pass's state is forgotten and, where its outputs
+// may come from the recurrences, G as the operand image of the tensor cores -- two halves of 32 samples, 32 rows of 128 bytes
+// each: rows 0..15 the words' TF32 values rounded to nearest, rows 16..31 the rounded remainders, 16-byte
+// chunk j of a row at chunk j ^ (row mod 8).  Otherwise the operands are the tensor-core kernel's (tc: the
+// pass's tables of that kernel).
+sos_status build_strip(sos_filter *f, LanePass &ps, LanePass &tc, double noise) {
     constexpr int N = 64;
     const int kp = ps.kp, S = 2 * kp;
     std::vector<float> buf(sosk::kStripImgFloats + static_cast<size_t>(S) * N, 0.f);
@@ -766,11 +780,20 @@ sos_status build_strip(sos_filter *f, LanePass &ps) {
             buf[sosk::kStripImgFloats + static_cast<size_t>(s) * N + j] = static_cast<float>(z[s]);
         }
     }
-    ps.warm_rows = strip_memory(ps.M1);
     ps.gresp.assign(buf.begin() + sosk::kStripImgFloats, buf.end());
-    if (cudaMalloc(&ps.d_strip, buf.size() * sizeof(float)) != cudaSuccess) return SOS_ENOMEM;
-    if (cudaMemcpy(ps.d_strip, buf.data(), buf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
-        return SOS_ECUDA;
+    ps.warm_rows = strip_memory(ps.M1);
+    tc.products = kp > sosk::kStripStatesK;
+    ps.products = tc.products && noise >= kStripProductsNoise;
+    if (!ps.products) {
+        if (cudaMalloc(&ps.d_strip, sizeof(float) * sosk::kStripImgFloats) != cudaSuccess) return SOS_ENOMEM;
+        if (cudaMemcpy(ps.d_strip, buf.data(), sizeof(float) * sosk::kStripImgFloats, cudaMemcpyHostToDevice) != cudaSuccess)
+            return SOS_ECUDA;
+    }
+    ps.gimg = ps.products ? tc.d_tcimg : ps.d_strip;
+    tc.gimg = tc.products ? tc.d_tcimg : ps.d_strip;
+    ps.gtail = tc.gtail = tc.d_gtail;
+    tc.warm_rows = ps.warm_rows;
+    tc.gresp = ps.gresp;
     return SOS_OK;
 }
 
@@ -1092,8 +1115,9 @@ sos_status launch_lane_pass(sos_filter *f, LanePass &ps, const float *x, float *
     p->aligned = aligned ? 1 : 0;
     p->tab = ps.d_tab;
     if (N == 64 && (TC || W == sosk::kLaneW)) {
-        p->gimg = ps.d_strip;
-        p->gtail = ps.d_strip ? ps.d_strip + sosk::kStripImgFloats : nullptr;
+        p->products = ps.products ? 1 : 0;
+        p->gimg = ps.gimg;
+        p->gtail = ps.gtail;
         p->gresp = ps.gresp.data();
         p->warm_rows = ps.warm_rows;
         p->norm = f->norm ? 1 : 0;
@@ -1880,13 +1904,11 @@ sos_status sos_filter_create(int n_sections, const double *sos, const float *zi,
     for (int i = 0; i < 4 && st == SOS_OK; ++i)
         st = build_lane(f, i == 0 ? 32 : 64, i == 2 ? sosk::kLaneWide : i == 3 ? sosk::kTcGroups : sosk::kLaneW,
                         f->lane[i]);
-    const bool strips = float32_noise(f) <= kStripNoise;
+    const double noise = float32_noise(f);
+    const bool strips = noise <= kStripNoise;
     for (size_t i = 0; i < f->lane[3].size() && st == SOS_OK; ++i) {
-        st = build_tc(f, f->lane[3][i]);
-        if (st == SOS_OK && strips) st = build_strip(f, f->lane[1][i]);
-        f->lane[3][i].d_strip = f->lane[1][i].d_strip;
-        f->lane[3][i].warm_rows = f->lane[1][i].warm_rows;
-        f->lane[3][i].gresp = f->lane[1][i].gresp;
+        st = build_tc(f, f->lane[3][i], strips);
+        if (st == SOS_OK && strips) st = build_strip(f, f->lane[1][i], f->lane[3][i], noise);
     }
     if (st == SOS_OK) {
         for (int g = 0; g < sosk::kBatchGeoms; ++g) {

@@ -141,6 +141,9 @@ constexpr int kStripUnit = 8192;        // samples of a unit of its work: 128 ro
 constexpr int kStripMax = 256;          // strips of a run (at most one per SM)
 constexpr size_t kStripTailBytes = 128 + 4 * kStripMax;  // a run's workspace, zero between runs
 constexpr int kStripImgFloats = 2048;   // tensor-core image of the state responses (8 KB)
+// up to this many sections the outputs come from the recurrences (2^28 samples at order 2: 330 to 360 us,
+// 88 to 96 % of the measured HBM rate); beyond, from the tensor cores too (LaneParams::products)
+constexpr int kStripStatesK = 2;
 
 // Per-section constants of the skewed-pass kernel, in the kernel's domain (b / b0 and b0 = 1 when
 // normalized; carried state = zscale * true state).
@@ -173,12 +176,13 @@ struct LaneParams {
     // blocks (k, j), j < k, of the lane transition M_N, row-major 2x2 at k (k - 1) / 2 + j
     float4 MX[K > 1 ? K * (K - 1) / 2 : 1];
     float A_tail[2 * K * (K + 1)];  // packed cascade transition over m_last + 1 samples
-    // the strip kernel's (kernels at N = 64): state responses as the tensor cores' operand image and in
-    // float32 ([2K][64]), rows of 64 samples until the cascade's state is forgotten in float32 (0: not
-    // within 2^14), workspace (nullptr: none), b0-normalized
+    // the strip kernel's (kernels at N = 64): the tensor cores' operand image (kStripImgFloats or, with
+    // outputs, kTcImageBytes) and the state responses in float32 ([2K][64]), rows of 64 samples until the cascade's state is forgotten in float32 (0: not
+    // within 2^14), whether the tensor cores form the outputs, b0-normalized, workspace (nullptr: none)
     const float *gimg, *gtail;
     const float *gresp;  // gtail in host memory
     int warm_rows;
+    int products;
     int norm;
     unsigned *tail;
 };

@@ -27,7 +27,7 @@
 //
 // Warp roles (one block per SM; the first eight warps give registers to the others):
 //   warps 0, 2, 3  load the units' samples (cp.async, zero-filled past the end, any alignment)
-//   warp 1         tensor-memory owner; lane 0 issues the products
+//   warp 1         tensor-memory owner; issues the products
 //   warps 4-7      split the rows into the products' operands, in tensor memory (two buffers)
 //   warps 8 on     three or four warpgroups, one unit each in turn; warp q of a warpgroup takes rows
 //                  32q .. 32q+31
@@ -35,6 +35,7 @@
 // Every wait is bounded by the spin budget.
 #pragma once
 #include <atomic>
+#include <cstring>
 
 #include "sosfilt_lane.cuh"
 #include "sosfilt_tcgen05.cuh"
@@ -46,45 +47,64 @@ constexpr int kStripRows = 128;                    // rows per unit (four groups
 static_assert(kStripUnit == kStripN * kStripRows, "unit geometry");
 constexpr int kStripXBytes = kStripUnit * 4;       // one staged unit: two column halves of 16 KB
 constexpr int kStripHalf = kStripXBytes / 2;
-constexpr int kStripCols = 64;                     // accumulator columns of a unit
-constexpr int kStripDS = 4;                        // accumulator slots: columns 0 .. 255
-constexpr int kStripACol = kStripDS * kStripCols;  // operand buffers: two of 64 + 64 columns behind them
-constexpr int kStripImg = 8192;                    // G image: two K halves of 32 rows x 128 B
+constexpr int kStripDS = 4;                        // accumulator slots, ahead of the operand buffers
 constexpr int kStripZ = 8;                         // units' incoming states kept (more than are in hand)
 constexpr int kStripBars = 384;                    // bytes of barriers and shared words
 constexpr long long kStripDrain = 2000000000LL;    // cycles a block waits for its own products at exit
 
-template <int K, bool TC_>
+// What the tensor cores do for a unit.
+enum StripMode {
+    kStripFma = 0,       // nothing: terminal states by FMAs, outputs by the recurrences
+    kStripStates = 1,    // terminal states; outputs by the recurrences
+    kStripOutputs = 2    // terminal states and outputs
+};
+
+template <int K, int MODE>
 struct StripDims {
     using Dm = LaneDims<K, kStripN, kLaneW>;
     static constexpr int S = 2 * K;
-    // epilogue warpgroups, and the registers a thread of the first two warpgroups (SREGS) and of theirs
-    // (REGS) has: four with 88 (768 threads of 80 at launch: 256 x 64 + 512 x 88), or three with 128 where
-    // the scan and the recurrences of five and more sections need them (640 threads of 96 at launch:
-    // 256 x 48 + 384 x 128)
-    static constexpr int WGS = K <= 4 ? 4 : 3;
-    static constexpr int SREGS = K <= 4 ? 64 : 48;
-    static constexpr int REGS = K <= 4 ? 88 : 128;
+    static constexpr bool TC = MODE != kStripFma, MM = MODE == kStripOutputs;
+    // epilogue warpgroups, and the registers that a thread of the first two warpgroups (SREGS) and of theirs
+    // (REGS) then has: 256 x 64 + 512 x 88 or 256 x 48 + 512 x 96 of 768 x 80 at launch; the recurrences of five
+    // and more sections want 128: 256 x 48 + 384 x 128 of 640 x 96 (four warpgroups with 96: 5 % slower)
+    static constexpr int WGS = MM || K <= 4 ? 4 : 3;
+    static constexpr int SREGS = MM || K > 4 ? 48 : 64;
+    static constexpr int REGS = MM ? 96 : K <= 4 ? 88 : 128;
     static constexpr int THREADS = 256 + 128 * WGS;
-    // terminal states on the tensor cores (else by FMAs: 128 or 256 a row, which one or two sections have
-    // the issue slots for, and which spare the signal's first unit the operands and products)
-    static constexpr bool TC = TC_;
     static constexpr int LOADERS = TC ? 3 : 8;  // loading warps
     static constexpr int U = TC ? 1 : 8;        // chunks of the recurrences unrolled
-    // shared memory after the staged units: G image, then floats: (M_N)^lane, (A_C)^v for v = 1 .. 4, the
-    // warpgroups' local carries (two slots), group states, unit states; then the barriers
+    // tensor memory: four accumulator slots (states only: two sets of 16 + 16 columns for the large and the
+    // small terms; outputs: 64, the terminal states' 16 and, in their place later, the row states' operand
+    // of 16 + 16), then the samples' operands, one buffer for each half of the rows (32 columns of heads and 32
+    // of remainders: while a half is multiplied the other is written)
+    static constexpr int COLS = MM ? 96 : 64;
+    static constexpr int ACOL = kStripDS * COLS;
+    static_assert(ACOL + 2 * 64 <= 512, "tensor memory");
+    // shared memory: staged units, operand image, the output staging (half a row for each of a
+    // warp's rows), then floats: (M_N)^b for b = 0 .. 7 and 8, 16, 24, (A_C)^v for v = 1 .. 4, the warpgroups' local carries (two slots), group states, unit states;
+    // and the barriers
+    // the operand image in shared memory; with outputs, of [T | G]'s second column half only rows 32 .. 79,
+    // the others being zeros that no product takes
+    static constexpr int B1 = (80 + 48) * 128;  // heads or remainders of [T | G]
+    static constexpr int IMG = MM ? 2 * B1 + 64 * 128 : 4 * kStripImgFloats;
+    static constexpr int STAGE = MM ? 4 * WGS * 4096 : 0;
+    
     static constexpr int T_ML = 0;
-    static constexpr int T_ACP = T_ML + 32 * Dm::MS;
+    static constexpr int T_ACP = T_ML + 11 * Dm::MS;
     static constexpr int T_A = T_ACP + 4 * S * S;
     static constexpr int T_ZV = T_A + WGS * 2 * 4 * S;
-    static constexpr int T_Z = T_ZV + WGS * 4 * S;
-    static constexpr int T_END = T_Z + kStripZ * S;
-    static constexpr int FIXED = kStripImg + 4 * T_END + kStripBars;
+    static constexpr int T_Z = T_ZV + WGS * 4 * 4 * S;
+    // the output basis H [S][64] and the states of the signal's first group (row_part), strip 0 only
+    static constexpr int T_H = T_Z + kStripZ * S;
+    static constexpr int T_ST = T_H + kStripN * S;
+    static constexpr int T_END = T_ST + (MM ? 0 : 32 * S);
+    static constexpr int FIXED = IMG + STAGE + 4 * T_END + kStripBars;
     static constexpr int XS_FIT = (227 * 1024 - FIXED) / kStripXBytes;
     static constexpr int XS = XS_FIT > 6 ? 6 : XS_FIT;  // staged units
-    static_assert(XS >= WGS + 2, "units in the epilogue and two loading");
+    static_assert(XS >= (MM ? 3 : WGS + 2), "units in the epilogue (with outputs: in the products) and two loading");
     static constexpr int OFF_IMG = XS * kStripXBytes;
-    static constexpr int OFF_TAB = OFF_IMG + kStripImg;
+    static constexpr int OFF_STAGE = OFF_IMG + IMG;
+    static constexpr int OFF_TAB = OFF_STAGE + STAGE;
     static constexpr int OFF_BAR = OFF_TAB + 4 * T_END;
     static constexpr size_t SMEM = OFF_BAR + kStripBars;
 };
@@ -135,14 +155,23 @@ inline bool strip_cut(long long n, int warm_rows, StripCut &c) {
 // longer ones on the tensor cores (2^28 samples at order 2: 329 us against 354).
 constexpr int kStripFmaRows = 4 * kStripRows;
 
-template <int K, bool TC>
+// Rows of the shortest signals of three and more sections taken by strips, and of three or four unaligned.
+constexpr long long kStripLeastRows = 2048, kStripLeastRows4 = 45000;
+// Strips of at least this many rows take TMA copies.
+constexpr int kStripTmaRows = 4 * kStripRows;
+// A signal's full rows of 64 samples as a tensor map, copied in boxes of 32 x box_rows (sosfilt_tc.cu).
+bool strip_rows_map(CUtensorMap *tm, const float *base, long long rows, int box_rows);
+
+template <int K, int MODE>
 struct StripParams {
     LaneParams<K> p;
     StripCut cut;
     int in_place;      // y == x: a strip's tail is stored once the next strip has read it
     int x_aligned, y_aligned;  // 16-byte aligned
+    int tma;           // tmx and tmy are set: full units are loaded, full groups' outputs stored by TMA
+    CUtensorMap tmx, tmy;  // x and y as [rows][64], boxes of 32 x 128 and 32 x 32, 128-byte swizzle
     unsigned long long host_tickets;  // what the host adds to the lookback kernels' ticket base
-    float g[TC ? 1 : 2 * K][kStripN];  // without the tensor cores: the state responses
+    float g[MODE == kStripFma ? 2 * K : 1][kStripN];  // without the tensor cores: the state responses
 };
 
 __device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned parity) {
@@ -158,6 +187,15 @@ __device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned pari
 // mbar_wait whose hardware suspension is never longer than the budget.
 __device__ __forceinline__ bool strip_wait1(unsigned long long *bar, unsigned parity, long long budget, int *status) {
     if (mbar_test(bar, parity)) return true;
+    if (budget < kSuspendHintNs / 2) {  // a budget below a suspension: no suspension
+        const long long t0 = clock64();
+        while (!mbar_test(bar, parity))
+            if (clock64() - t0 > budget) {
+                atomicOr(status, kDevErrTimeout);
+                return false;
+            }
+        return true;
+    }
     const unsigned hint = budget < kSuspendHintNs ? static_cast<unsigned>(budget) : kSuspendHintNs;
     const long long t0 = clock64();
     while (!mbar_try_wait_sleep(bar, parity, hint)) {
@@ -331,6 +369,74 @@ __device__ __forceinline__ void lane_recurrence(const Secs &cs, unsigned char *s
     }
 }
 
+// The signal's first group: an initial state may be thousands of times the outputs that are left of it, and 64
+// steps of the recurrences from it err by as many roundings of the coefficients; so there the recurrences run
+// from zero state and the state's part (Eq. 24) is added from the output basis H ([2K][64], float64-derived),
+// both in shared memory.
+template <int K>
+__device__ __forceinline__ void row_part(unsigned char *sm, unsigned row, const float *H, const float *st) {
+#pragma unroll(K <= 2 ? 8 : 2)
+    for (int j = 0; j < kStripN / 4; ++j) {
+        float4 *a = reinterpret_cast<float4 *>(sm + (row ^ ((j & 7) << 4)) + (j >> 3) * kStripHalf);
+        float4 v = *a;
+#pragma unroll
+        for (int s = 0; s < 2 * K; ++s) {
+            const float4 b = *reinterpret_cast<const float4 *>(H + s * kStripN + 4 * j);
+            const float z = st[s];
+            v.x = fmaf(b.x, z, v.x);
+            v.y = fmaf(b.y, z, v.y);
+            v.z = fmaf(b.z, z, v.z);
+            v.w = fmaf(b.w, z, v.w);
+        }
+        *a = v;
+    }
+}
+
+// A chunk of four samples k .. k + 3 of a group whose own samples are from .. to - 1 (from a multiple of four).
+__device__ __forceinline__ void put4(float *y, int k, int from, int to, const float4 &v) {
+    if (k >= from && k + 4 <= to) {
+        __stcs(reinterpret_cast<float4 *>(y + k), v);
+    } else if (k >= from) {
+        if (k + 0 < to) y[k] = v.x;
+        if (k + 1 < to) y[k + 1] = v.y;
+        if (k + 2 < to) y[k + 2] = v.z;
+    }
+}
+
+// The `count` samples of the row at sample `at`, by the sections one after the other from the row's state
+// (transposed direct form II), from the signal to the output directly.  For rows whose products are worth
+// nothing: rare, and small rather than fast.
+template <int K>
+__device__ __noinline__ void row_plainly(const LaneParams<K> &p, long long at, int count, const float (&st)[16]) {
+    float z[2 * K];
+    for (int s = 0; s < 2 * K; ++s) z[s] = st[s];
+    for (int m = 0; m < count; ++m) {
+        float v = p.x[at + m] * p.gain;
+        for (int s = 0; s < K; ++s) {
+            const float4 c = p.sec[s].c;  // b1, b2, -a1, -a2
+            const float y = fmaf(p.sec[s].b0, v, z[2 * s]);
+            z[2 * s] = fmaf(c.x, v, fmaf(c.z, y, z[2 * s + 1]));
+            z[2 * s + 1] = fmaf(c.y, v, c.w * y);
+            v = y;
+        }
+        p.y[at + m] = v;
+    }
+}
+
+// Row `row` of y = A x, A dense column-major S x S and x in shared memory (read as pairs, broadcast): no
+// shuffles, so that products of several vectors overlap.
+template <int S>
+__device__ __forceinline__ float mv_shared(const float *A, const float *x, int row) {
+    float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < S; j += 2) {
+        const float2 v = *reinterpret_cast<const float2 *>(x + j);
+        y0 = fmaf(A[j * S + row], v.x, y0);
+        y1 = fmaf(A[(j + 1) * S + row], v.y, y1);
+    }
+    return y0 + y1;
+}
+
 // Words of the run's workspace (LaneParams::tail), all zero between runs.
 struct StripTail {
     unsigned ticket, poison, done, pad;
@@ -342,14 +448,14 @@ static_assert(sizeof(StripTail) <= kStripTailBytes, "workspace of a run");
 // Barriers of a block: staged units, operand buffers, accumulator slots, units' incoming states.
 template <int XS>
 struct StripBars {
-    unsigned long long full[XS], xfree[XS], afull[2], afree[2], dfull[kStripDS], dfree[kStripDS], zready[kStripZ], fin;
+    unsigned long long full[XS], xfree[XS], afull[2], afree[2], dfull[kStripDS], dfree[kStripDS], zready[kStripZ], yfull[4], fin;
     unsigned tmem, strip, last, pad;
 };
 
-template <int K, bool NORM, bool TC>
-__global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
-    sos_strip_kernel(const __grid_constant__ StripParams<K, TC> P) {
-    using Sd = StripDims<K, TC>;
+template <int K, bool NORM, int MODE>
+__global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
+    sos_strip_kernel(const __grid_constant__ StripParams<K, MODE> P) {
+    using Sd = StripDims<K, MODE>;
     using Dm = typename Sd::Dm;
     constexpr int S = Sd::S, MS = Dm::MS, XS = Sd::XS, WGS = Sd::WGS;
     const LaneParams<K> &p = P.p;
@@ -384,6 +490,7 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
             mbar_init(&dfree[i], 4);
         }
         for (int i = 0; i < kStripZ; ++i) mbar_init(&zready[i], 1);
+        for (int i = 0; i < 4; ++i) mbar_init(&bars.yfull[i], 1);
         mbar_init(&bars.fin, 1);
     }
     if (Sd::TC && warp == 1) tc_alloc512(&bars.tmem);
@@ -415,12 +522,26 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
         if constexpr (Sd::TC) {
             const float4 *src = reinterpret_cast<const float4 *>(p.gimg);
             float4 *dst = reinterpret_cast<float4 *>(sm + Sd::OFF_IMG);
-            for (int i = k; i < kStripImg / 16; i += step) dst[i] = __ldg(src + i);
+            if constexpr (Sd::MM) {
+                constexpr int HALF = 80 * 8, SKIP = 32 * 8;  // 16-byte words of a column half, and of its zeros
+                for (int i = k; i < 4 * HALF; i += step) {   // heads, then remainders, two halves each
+                    const int part = i / HALF, w = i % HALF, odd = part & 1;
+                    if (!odd) dst[(part >> 1) * (Sd::B1 / 16) + w] = __ldg(src + i);
+                    else if (w >= SKIP) dst[(part >> 1) * (Sd::B1 / 16) + HALF + w - SKIP] = __ldg(src + i);
+                }
+                for (int i = k; i < 64 * 8; i += step) dst[2 * Sd::B1 / 16 + i] = __ldg(src + 4 * HALF + i);
+            } else {
+                for (int i = k; i < Sd::IMG / 16; i += step) dst[i] = __ldg(src + i);
+            }
         }
-        for (int i = k; i < 32 * MS / 4; i += step)
-            reinterpret_cast<float4 *>(sML)[i] = __ldg(reinterpret_cast<const float4 *>(p.tab) + i);
+        for (int i = k; i < 11 * MS / 4; i += step) {
+            const int m = i / (MS / 4), lane_of = m < 8 ? m : 8 * (m - 7);
+            reinterpret_cast<float4 *>(sML)[i] = __ldg(reinterpret_cast<const float4 *>(p.tab) + lane_of * (MS / 4) + i % (MS / 4));
+        }
         for (int i = k; i < 4 * S * S; i += step) sACp[i] = __ldg(p.tab + Dm::OFF_ACP + i);
-        if (Sd::TC) fence_proxy_async_smem();  // the G image is read by the tensor cores
+        if (p.zi && r_first == 0)
+            for (int i = k; i < kStripN * S; i += step) tabs[Sd::T_H + i] = __ldg(p.tab + Dm::OFF_H + i);
+        if (Sd::TC) fence_proxy_async_smem();  // the image is read by the tensor cores
         named_bar_sync(8, step);
         if (warp == 8) trace(0, 21);
     };
@@ -442,6 +563,18 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
             const long long avail = (r_end * kStripN < p.n ? r_end * kStripN : p.n) - base;
             const float *x = p.x + base;
             const unsigned dst = smem_u32(sm) + xs * kStripXBytes;
+            if (P.tma && avail >= kStripUnit) {
+                if (w == 0 && lane == 0) {
+                    mbar_expect_tx(&full[xs], kStripXBytes);
+                    const long long row = r_first + static_cast<long long>(i) * kStripRows;
+                    tma_load_2d(sm + xs * kStripXBytes, &P.tmx, 0, row, &full[xs]);
+                    tma_load_2d(sm + xs * kStripXBytes + kStripHalf, &P.tmx, 32, row, &full[xs]);
+                } else {
+                    mbar_arrive(&full[xs]);
+                }
+                if (w == 0) trace(i, 16);
+                continue;
+            }
             if (P.x_aligned) {
                 // 16-byte copies: lane = (row parity, chunk of the row); row 8m + 2k + parity has the chunk at
                 // (chunk ^ parity ^ 2k) & 7
@@ -484,72 +617,99 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
     } else if (Sd::TC && warp == 1) {
         // ------------------------------------------------------------------ products
         load_tables();
-        if (lane == 0) {
-            constexpr unsigned i32 = tc_idesc(32), i16 = tc_idesc(16);
-            const unsigned g = smem_u32(sm + Sd::OFF_IMG);
+        {
+            const unsigned g = smem_u32(sm + Sd::OFF_IMG), go = tc_elect();
             for (unsigned i = 0; i < n_u; ++i) {
-                const unsigned ds = i % kStripDS, b = i & 1;
-                if (i >= kStripDS && !strip_wait1(&dfree[ds], (i / kStripDS - 1) & 1, budget, p.status)) break;
-                if (!strip_wait1(&afull[b], (i >> 1) & 1, budget, p.status)) break;
-                tc_fence_after();
-                trace(i, 17);
-                const unsigned d = tmem + ds * kStripCols, xa = tmem + kStripACol + b * 128, lo = xa + 64;
-                // x [G_hi | G_lo]: columns 0..31 over the first half of the row, 32..63 over the second; the
-                // remainder's products join the small terms, columns 16..31
+                const unsigned ds = i % kStripDS;
+                if (i >= kStripDS && !strip_wait(&dfree[ds], (i / kStripDS - 1) & 1, budget, p.status)) break;
+                const unsigned d = tmem + ds * Sd::COLS;
+                bool ok = true;
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const unsigned gk = g + (k >> 2) * (kStripImg / 2) + (k & 3) * 32;
-                    tc_mma_ts(d + 32 * (k >> 2), xa + 8 * k, tc_sdesc(gk), i32, (k & 3) ? 1u : 0u);
-                    tc_mma_ts(d + 16, lo + 8 * k, tc_sdesc(gk), i16, 1u);
-                    tc_mma_ts(d + 16, lo + 8 * k, tc_sdesc(gk + 16 * 128), i16, 1u);
+                for (int h = 0; h < 2; ++h) {  // half of the rows' samples at a time
+                    ok = ok && strip_wait(&afull[h], i & 1, budget, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (h == 0) trace(i, 17);
+                    const unsigned hi = tmem + Sd::ACOL + 64 * h, lo = hi + 32;
+                    if constexpr (Sd::MM) {
+                        // [Y_p | T] = X [T^T | G^T]: columns 0..63 the rows' zero-state outputs, 64..79 their
+                        // terminal states.  T is lower triangular, so the samples from 16 j on enter columns
+                        // 16 j .. only.  The small terms first
+                        auto chain = [&](unsigned a, int image, bool first) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int off = 32 * h + 16 * (k >> 1);
+                                tc_mma_ts(d + off, a + 8 * k, tc_sdesc(g + image + (h ? 80 + off - 32 : off) * 128 + k * 32),
+                                          tc_idesc(80 - off), first && h == 0 && k == 0 ? 0u : 1u, go);
+                            }
+                        };
+                        chain(lo, 0, true);        // remainders of x, heads of the image
+                        chain(hi, Sd::B1, false);  // heads of x, remainders of the image
+                        chain(hi, 0, false);       // heads of both
+                    } else {
+                        // x [G_hi | G_lo]: columns 32 h .. 32 h + 31; the remainders' products join the small
+                        // terms, columns 16..31
+                        constexpr unsigned i32 = tc_idesc(32), i16 = tc_idesc(16);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const unsigned gk = g + h * (Sd::IMG / 2) + k * 32;
+                            tc_mma_ts(d + 32 * h, hi + 8 * k, tc_sdesc(gk), i32, k ? 1u : 0u, go);
+                            tc_mma_ts(d + 16, lo + 8 * k, tc_sdesc(gk), i16, 1u, go);
+                            tc_mma_ts(d + 16, lo + 8 * k, tc_sdesc(gk + 16 * 128), i16, 1u, go);
+                        }
+                    }
+                    tc_commit_if(&afree[h], go);
                 }
-                tc_commit(&afree[b]);
-                tc_commit(&dfull[ds]);
+                if (!ok) break;
+                tc_commit_if(&dfull[ds], go);
                 trace(i, 18);
             }
             // every product issued has completed before tensor memory is released
-            tc_commit(&bars.fin);
-            strip_wait1(&bars.fin, 0, kStripDrain, p.status);
+            __syncwarp();
+            tc_commit_if(&bars.fin, go);
+            strip_wait(&bars.fin, 0, kStripDrain, p.status);
         }
-        __syncwarp();
     } else {
         // ------------------------------------------------------------------ operands of the products
         load_tables();
         const int r = 32 * (warp - 4) + lane;  // row within the unit
-        const unsigned ta = tmem + kStripACol + (static_cast<unsigned>(32 * (warp - 4)) << 16);
-        // the remainder x - (upper 19 bits of x) is exact in 13 bits; half a unit of the 11 the tensor
-        // core reads is added to its magnitude, so that the cut rounds to nearest
-        auto rem = [](float x) {
-            const float e = x - __uint_as_float(__float_as_uint(x) & 0xffffe000u);
-            return __uint_as_float(__float_as_uint(e) + 0x1000u);
-        };
+        const unsigned ta = tmem + Sd::ACOL + (static_cast<unsigned>(32 * (warp - 4)) << 16);
+        // heads: the nearest TF32 values; remainders: exact in 12 bits, of which the tensor core reads 11
         for (unsigned i = 0; i < n_u; ++i) {
-            const unsigned xs = i % XS, b = i & 1;
+            const unsigned xs = i % XS;
             if (!strip_wait(&full[xs], (i / XS) & 1, budget, p.status)) break;
             if (warp == 4) trace(i, 1);
             if (P.in_place && warp == 4 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows) {
                 __threadfence();
                 atomicExch(&tail->flag[strip], 1u);  // the warm-up samples have been read
             }
-            if (i >= 2 && !strip_wait(&afree[b], ((i >> 1) - 1) & 1, budget, p.status)) break;
-            tc_fence_after();
-            if (warp == 4) trace(i, 2);
             const unsigned char *X = sm + xs * kStripXBytes + r * 128;
-            const unsigned t0 = ta + b * 128;
-#pragma unroll 2
-            for (int j = 0; j < 8; ++j) {  // eight samples at a time
-                const unsigned char *h = X + (j >> 2) * kStripHalf;
-                const int c = 2 * (j & 3);
-                const float4 u = *reinterpret_cast<const float4 *>(h + ((c ^ (r & 7)) << 4));
-                const float4 v = *reinterpret_cast<const float4 *>(h + (((c + 1) ^ (r & 7)) << 4));
-                tc_st8(t0 + 8 * j, u, v);
-                tc_st8(t0 + 64 + 8 * j, make_float4(rem(u.x), rem(u.y), rem(u.z), rem(u.w)),
-                       make_float4(rem(v.x), rem(v.y), rem(v.z), rem(v.w)));
+            bool ok = true;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                ok = ok && (i == 0 || strip_wait(&afree[h], (i - 1) & 1, budget, p.status));
+                if (!ok) break;
+                tc_fence_after();
+                if (warp == 4 && h == 0) trace(i, 2);
+                const unsigned char *Xh = X + h * kStripHalf;
+                const unsigned t0 = ta + 64 * h;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {  // eight samples at a time
+                    const float4 u = *reinterpret_cast<const float4 *>(Xh + (((2 * j) ^ (r & 7)) << 4));
+                    const float4 v = *reinterpret_cast<const float4 *>(Xh + (((2 * j + 1) ^ (r & 7)) << 4));
+                    const float4 uh = make_float4(tf32_near(u.x), tf32_near(u.y), tf32_near(u.z), tf32_near(u.w));
+                    const float4 vh = make_float4(tf32_near(v.x), tf32_near(v.y), tf32_near(v.z), tf32_near(v.w));
+                    tc_st8(t0 + 8 * j, uh, vh);
+                    tc_st8(t0 + 32 + 8 * j, make_float4(u.x - uh.x, u.y - uh.y, u.z - uh.z, u.w - uh.w),
+                           make_float4(v.x - vh.x, v.y - vh.y, v.z - vh.z, v.w - vh.w));
+                }
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&afull[h]);
             }
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&afull[b]);
+            if (!ok) break;
+            if (Sd::MM && lane == 0) mbar_arrive(&xfree[xs]);
             if (warp == 4) trace(i, 3);
         }
     }
@@ -561,14 +721,16 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
         const int r = 32 * q + lane;  // row within the unit
         const unsigned tl = tmem + (static_cast<unsigned>(32 * q) << 16);
         const ParamSecs<K> cs{p};
-        float *zv = tabs + Sd::T_ZV + (wg * 4 + q) * S;
+        float *zv = tabs + Sd::T_ZV + (wg * 4 + q) * 4 * S;  // [4][S]
         const int li = lane < S ? lane : 0;
         bool dead = false;
-        unsigned par = 0;
+        unsigned par = 0, y_par = 0;
         for (unsigned i = wg; i < n_u; i += WGS, par ^= 1) {
             const unsigned ds = i % kStripDS, xs = i % XS;
             float *ab = tabs + Sd::T_A + (wg * 2 + par) * 4 * S;
             float Sl[S];
+            [[maybe_unused]] bool released = false;  // the accumulator slot
+            bool bad = false;  // the row's samples are not all finite (its products are then worth nothing)
             bool ok = !dead && (Sd::TC ? strip_wait(&dfull[ds], (i / kStripDS) & 1, budget, p.status)
                                        : strip_wait(&full[xs], (i / XS) & 1, budget, p.status));
             const long long R = r_first + static_cast<long long>(i) * kStripRows + 32 * q;  // the warp's first row
@@ -595,17 +757,26 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                     }
 #pragma unroll
                     for (int s = 0; s < S; ++s) t[s] = a[s][0] + a[s][1];
+                } else if constexpr (Sd::MM) {
+                    tc_fence_after();
+                    constexpr int C = S <= 2 ? 2 : S <= 4 ? 4 : S <= 8 ? 8 : 16;
+                    float a[C];
+                    tc_ldn<C>(tl + ds * Sd::COLS + 64, a);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < S; ++j) t[j] = a[j];
+                    bad = !(fabsf(t[0]) <= 3.402823466e38f);
                 } else {
                     tc_fence_after();
                     constexpr int C = S <= 2 ? 2 : S <= 4 ? 4 : S <= 8 ? 8 : 16;
                     float a0[C], a1[C];
-                    tc_ldn<C>(tl + ds * kStripCols + 16, a0);  // the small terms
-                    tc_ldn<C>(tl + ds * kStripCols + 48, a1);
+                    tc_ldn<C>(tl + ds * Sd::COLS + 16, a0);  // the small terms
+                    tc_ldn<C>(tl + ds * Sd::COLS + 48, a1);
                     tc_wait_ld();
 #pragma unroll
                     for (int j = 0; j < S; ++j) t[j] = a0[j] + a1[j];
-                    tc_ldn<C>(tl + ds * kStripCols, a0);
-                    tc_ldn<C>(tl + ds * kStripCols + 32, a1);
+                    tc_ldn<C>(tl + ds * Sd::COLS, a0);
+                    tc_ldn<C>(tl + ds * Sd::COLS + 32, a1);
                     tc_wait_ld();
 #pragma unroll
                     for (int j = 0; j < S; ++j) t[j] = (a0[j] + a1[j]) + t[j];
@@ -620,20 +791,22 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
             if (!named_bar_and(1 + wg, 128, ok)) break;
             // the fold's prefix p_v (carry of the groups before this warp's under zero state), then, once
             // the unit's incoming state is known, the group's: Z_v = (A_C)^v Z + p_v
-            float pv = 0.f;
-            if (q >= 1) pv = ab[li];
-#pragma unroll 1
-            for (int v = 1; v < q; ++v) pv = lane_mv<S>(sACp, pv, lane) + ab[v * S + li];
-            float cu = 0.f;
-            if (q == 3) cu = lane_mv<S>(sACp, pv, lane) + ab[3 * S + li];
-            if (!strip_wait(&zready[i % kStripZ], (i / kStripZ) & 1, budget, p.status)) {
-                dead = true;
-                continue;
-            }
-            if (q == 0) trace(i, 9);
-            const float z0 = z_buf[(i % kStripZ) * S + li];
+            // p_v = a_{v-1} + A_C a_{v-2} + (A_C)^2 a_{v-3} and the unit's carry c: independent products
+            const float *A1 = sACp, *A2 = sACp + S * S, *A3 = sACp + 2 * S * S, *A4 = sACp + 3 * S * S;
+            float pv = 0.f, cu = 0.f;
+            if (q == 1) pv = ab[li];
+            if (q == 2) pv = mv_shared<S>(A1, ab, li) + ab[S + li];
             if (q == 3) {
-                const float zn = lane_mv<S>(sACp + 3 * S * S, z0, lane) + cu;
+                pv = (mv_shared<S>(A2, ab, li) + mv_shared<S>(A1, ab + S, li)) + ab[2 * S + li];
+                cu = (mv_shared<S>(A3, ab, li) + mv_shared<S>(A2, ab + S, li)) +
+                     (mv_shared<S>(A1, ab + 2 * S, li) + ab[3 * S + li]);
+            }
+            dead = !strip_wait(&zready[i % kStripZ], (i / kStripZ) & 1, budget, p.status);
+            if (!Sd::MM && dead) continue;
+            if (q == 0) trace(i, 9);
+            const float *z0 = z_buf + (i % kStripZ) * S;
+            if (q == 3) {
+                const float zn = mv_shared<S>(A4, z0, li) + cu;
                 if (i + 1 < n_u) {
                     if (lane < S) z_buf[((i + 1) % kStripZ) * S + lane] = zn;
                     __syncwarp();
@@ -642,27 +815,57 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                     atomicMax(&tail->poison, static_cast<unsigned>(P.cut.n_strips - strip));
                 }
             }
-            if (R + 32 > r_own && R < r_end) {
-                const float zq = q == 0 ? z0 : lane_mv<S>(sACp + (q - 1) * S * S, z0, lane) + pv;
+            // the unit's first and last own rows; with outputs its four warps stay together for the products
+            const bool own = R + 32 > r_own && R < r_end;
+            const bool unit_own = R - 32 * q + kStripRows > r_own;
+            if (Sd::MM ? unit_own : own) {
+                const float zq = q == 0 ? z0[li] : mv_shared<S>(q == 1 ? A1 : q == 2 ? A2 : A3, z0, li) + pv;
+                // (M_N)^lane Z_v in two steps, lane = 8 a + b: the four (M_N)^(8 a) Z_v, a section's two words a
+                // lane, then each lane's (M_N)^b of one of them (11 matrices to read instead of 32)
                 if (lane < S) zv[lane] = zq;
+                __syncwarp();
+                {
+                    const int a = lane >> 3, s = lane & 7;
+                    float w0 = 0.f, w1 = 0.f;
+                    if (a > 0 && s < K) {
+                        const float *m = sML + (7 + a) * MS + 2 * s * (s + 1);
+#pragma unroll
+                        for (int j = 0; j < K; ++j)
+                            if (j <= s) {
+                                const float4 B = *reinterpret_cast<const float4 *>(m + 4 * j);
+                                const float2 z = *reinterpret_cast<const float2 *>(zv + 2 * j);
+                                w0 = fmaf(B.x, z.x, fmaf(B.y, z.y, w0));
+                                w1 = fmaf(B.z, z.x, fmaf(B.w, z.y, w1));
+                            }
+                        *reinterpret_cast<float2 *>(zv + a * S + 2 * s) = make_float2(w0, w1);
+                    }
+                }
                 __syncwarp();
                 float st[S];
 #pragma unroll
                 for (int j = 0; j < S; ++j) st[j] = Sl[j];
-                lane_state_mv<K>(sML + lane * MS, zv, st);
+                lane_state_mv<K>(sML + (lane & 7) * MS, zv + (lane >> 3) * S, st);
                 unsigned char *X = sm + xs * kStripXBytes;
+                const long long base = R * kStripN;
                 if (q == 0) trace(i, 10);
                 if (p.zf && r_end == P.cut.n_rows && R + 32 >= r_end) {
                     // final state: the last row's samples under zero state, taken across the lanes, plus
                     // the transition of the row's incoming state over them
                     const int lane_last = static_cast<int>(P.cut.n_rows - 1 - R);
-                    const int ml = p.m_last, rl = 32 * q + lane_last;
+                    const int ml = p.m_last;
+                    [[maybe_unused]] const int rl = 32 * q + lane_last;
                     float acc[S], zt[S];
                     {
                         const float *gt = p.gtail + (kStripN - 1 - ml);
-                        const float xa = lane <= ml ? *reinterpret_cast<const float *>(X + tc_swz(rl, lane)) : 0.f;
-                        const float xb =
-                            lane + 32 <= ml ? *reinterpret_cast<const float *>(X + kStripHalf + tc_swz(rl, lane)) : 0.f;
+                        float xa = 0.f, xb = 0.f;
+                        if constexpr (Sd::MM) {  // the stage is gone; the signal is still as it was here, in place too
+                            const float *xr = p.x + base + lane_last * kStripN;
+                            if (lane <= ml) xa = xr[lane];
+                            if (lane + 32 <= ml) xb = xr[lane + 32];
+                        } else {
+                            if (lane <= ml) xa = *reinterpret_cast<const float *>(X + tc_swz(rl, lane));
+                            if (lane + 32 <= ml) xb = *reinterpret_cast<const float *>(X + kStripHalf + tc_swz(rl, lane));
+                        }
 #pragma unroll
                         for (int s = 0; s < S; ++s) {
                             float v = lane <= ml ? __ldg(gt + s * kStripN + lane) * xa : 0.f;
@@ -684,10 +887,76 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                     }
                     __syncwarp();
                 }
-                lane_recurrence<K, NORM, Sd::U>(cs, sm, xs * kStripXBytes + r * 128 + ((r & 7) << 4), p.gain, st);
-                __syncwarp();
+                if constexpr (Sd::MM) {
+                    if (p.zi && r_first == 0 && i == 0 && q == 0 && !__any_sync(0xffffffffu, bad)) {
+                        // the signal's first group: its states' part is added in float32 (row_part; as operands of
+                        // 22 bits they would err by as much), and none are left to multiply.  (Rows that
+                        // are done plainly below take theirs from the operand.)
+                        const float *H = tabs + Sd::T_H;
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            float v[16];
+                            tc_ldn<16>(tl + ds * Sd::COLS + 16 * c, v);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int j = 0; j < S; ++j)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    const float4 b = *(reinterpret_cast<const float4 *>(H + j * kStripN + 16 * c) + k);
+                                    v[4 * k] = fmaf(b.x, st[j], v[4 * k]);
+                                    v[4 * k + 1] = fmaf(b.y, st[j], v[4 * k + 1]);
+                                    v[4 * k + 2] = fmaf(b.z, st[j], v[4 * k + 2]);
+                                    v[4 * k + 3] = fmaf(b.w, st[j], v[4 * k + 3]);
+                                }
+                            tc_st16(tl + ds * Sd::COLS + 16 * c, v);
+                        }
+#pragma unroll
+                        for (int j = 0; j < S; ++j) st[j] = 0.f;
+                    }
+                    // the rows' states as an operand beside the accumulator, then Y += St H^T, small terms first,
+                    // issued by the warpgroup's first warp
+                    float e[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) e[j] = j < S ? tf32_near(st[j < S ? j : 0]) : 0.f;
+                    tc_st16(tl + ds * Sd::COLS + 64, e);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) e[j] = j < S ? st[j < S ? j : 0] - e[j] : 0.f;
+                    tc_st16(tl + ds * Sd::COLS + 80, e);
+                    tc_wait_st();
+                    tc_fence_before();
+                    if (!named_bar_and(9 + wg, 128, !dead)) break;
+                    if (q == 0) {
+                        tc_fence_after();
+                        constexpr unsigned i64 = tc_idesc(64);
+                        const unsigned d = tmem + ds * Sd::COLS, h = smem_u32(sm + Sd::OFF_IMG) + 2 * Sd::B1, go = tc_elect();
+                        constexpr int KK = S > 8 ? 2 : 1;
+#pragma unroll
+                        for (int k = 0; k < KK; ++k) tc_mma_ts(d, d + 80 + 8 * k, tc_sdesc(h + 32 * k), i64, 1u, go);
+#pragma unroll
+                        for (int k = 0; k < KK; ++k) tc_mma_ts(d, d + 64 + 8 * k, tc_sdesc(h + 64 + 32 * k), i64, 1u, go);
+#pragma unroll
+                        for (int k = 0; k < KK; ++k) tc_mma_ts(d, d + 64 + 8 * k, tc_sdesc(h + 32 * k), i64, 1u, go);
+                        tc_commit_if(&bars.yfull[wg], go);
+                    }
+                    if (!strip_wait(&bars.yfull[wg], y_par, budget, p.status)) dead = true;
+                    y_par ^= 1;
+                    tc_fence_after();
+                } else {
+                    const unsigned row = xs * kStripXBytes + r * 128 + ((r & 7) << 4);
+                    const bool first = p.zi && r_first == 0 && i == 0 && q == 0;
+                    if (first) {
+#pragma unroll
+                        for (int j = 0; j < S; ++j) {
+                            tabs[Sd::T_ST + lane * S + j] = st[j];
+                            st[j] = 0.f;
+                        }
+                    }
+                    lane_recurrence<K, NORM, Sd::U>(cs, sm, row, p.gain, st);
+                    if (first) row_part<K>(sm, row, tabs + Sd::T_H, tabs + Sd::T_ST + lane * S);
+                    __syncwarp();
+                }
                 if (q == 0) trace(i, 11);
-                if (P.in_place && strip + 1 < P.cut.n_strips && R + 32 > r_end - P.cut.warm_rows) {
+                if (P.in_place && own && strip + 1 < P.cut.n_strips && R + 32 > r_end - P.cut.warm_rows) {
                     const long long t0 = clock64();
                     bool seen = false, late = false;
                     while (!seen && !late) {
@@ -697,17 +966,88 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                     if (!__all_sync(0xffffffffu, seen)) {
                         if (lane == 0) atomicOr(p.status, kDevErrTimeout);
                         dead = true;
-                        continue;
                     }
                 }
-                // the group's own samples: from .. to - 1, counted from its first row
-                const long long base = R * kStripN;
+                if (!Sd::MM && dead) continue;
+                // the group's own samples: from .. to - 1, counted from its first row (none of a group outside)
                 const int from = R < r_own ? static_cast<int>(r_own - R) * kStripN : 0;
                 const long long own_end = r_end * kStripN < p.n ? r_end * kStripN : p.n;
-                const int to = own_end - base < 32 * kStripN ? static_cast<int>(own_end - base) : 32 * kStripN;
+                const int to = !own ? 0 : own_end - base < 32 * kStripN ? static_cast<int>(own_end - base) : 32 * kStripN;
                 float *y = p.y + base;
-                const unsigned char *Xw = X + 32 * q * 128;
-                if (P.y_aligned) {
+                if constexpr (Sd::MM) {
+                    const unsigned bad_rows = __ballot_sync(0xffffffffu, bad);
+                    const unsigned sg = Sd::OFF_STAGE + (warp - 8) * 4096;  // 32 rows x 128 B, chunks permuted
+                    if (bad_rows && !dead) {
+                        // rows with samples that are not finite: the outputs up to the first of them are right
+                        // by the recurrence, which is run from the rows' states on the signal itself
+                        float e[16], l[16];
+                        tc_ldn<16>(tl + ds * Sd::COLS + 64, e);
+                        tc_ldn<16>(tl + ds * Sd::COLS + 80, l);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) e[j] += l[j];
+                        const int k = lane * kStripN;
+                        if (bad && k >= from && k < to) row_plainly<K>(p, base + k, to - k < kStripN ? to - k : kStripN, e);
+                        __syncwarp();
+                    }
+                    if (!dead) {
+                        float v[64];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) tc_ldn<16>(tl + ds * Sd::COLS + 16 * k, *reinterpret_cast<float(*)[16]>(v + 16 * k));
+                        tc_wait_ld();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&dfree[ds]);
+                        released = true;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {  // half a row at a time through the staging
+                            if (P.tma) {  // the last store has read it
+                                if (lane == 0) bulk_wait_read0();
+                                __syncwarp();
+                            }
+#pragma unroll
+                            for (int c = 0; c < 8; ++c)
+                                *reinterpret_cast<float4 *>(sm + sg + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+                                    make_float4(v[32 * h + 4 * c], v[32 * h + 4 * c + 1], v[32 * h + 4 * c + 2], v[32 * h + 4 * c + 3]);
+                            if (P.tma && from == 0 && to == 32 * kStripN && !bad_rows) {
+                                fence_proxy_async_smem();
+                                __syncwarp();
+                                if (lane == 0) {
+                                    tma_store_2d(&P.tmy, 32 * h, R, sm + sg);
+                                    bulk_commit();
+                                }
+                                continue;
+                            }
+                            __syncwarp();
+                            if (P.y_aligned) {
+                                const int c = lane & 7, r1 = lane >> 3;
+                                const int k0 = r1 * kStripN + 32 * h + 4 * c;
+                                auto get = [&](int j) {
+                                    const int rr = 4 * j + r1;
+                                    return *reinterpret_cast<const float4 *>(sm + sg + rr * 128 + ((c ^ (rr & 7)) << 4));
+                                };
+                                if (from == 0 && to == 32 * kStripN && !bad_rows) {
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) __stcs(reinterpret_cast<float4 *>(y + k0 + 4 * j * kStripN), get(j));
+                                } else {
+#pragma unroll 2
+                                    for (int j = 0; j < 8; ++j) {
+                                        const int k = k0 + 4 * j * kStripN;
+                                        if (!(bad_rows >> (4 * j + r1) & 1)) put4(y, k, from, to, get(j));
+                                    }
+                                }
+                            } else {
+#pragma unroll 4
+                                for (int j = 0; j < 32; ++j) {
+                                    const int k = j * kStripN + 32 * h + lane;
+                                    const float v = *reinterpret_cast<const float *>(sm + sg + tc_swz(j, lane));
+                                    if (k >= from && k < to && !(bad_rows >> j & 1)) __stcs(y + k, v);
+                                }
+                            }
+                            __syncwarp();
+                        }
+                    }
+                } else if (P.y_aligned) {
                     const int c = lane & 15, r1 = lane >> 4;
                     const unsigned src = xs * kStripXBytes + (32 * q + r1) * 128 + (c >> 3) * kStripHalf + (((c & 7) ^ r1) << 4);
                     const int k0 = r1 * kStripN + 4 * c;  // from is a multiple of 64
@@ -719,19 +1059,10 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                         for (int j = 0; j < 16; ++j) __stcs(reinterpret_cast<float4 *>(y + k0 + 2 * j * kStripN), get(j));
                     } else {
 #pragma unroll 4
-                        for (int j = 0; j < 16; ++j) {
-                            const int k = k0 + 2 * j * kStripN;
-                            const float4 v = get(j);
-                            if (k >= from && k + 4 <= to) {
-                                __stcs(reinterpret_cast<float4 *>(y + k), v);
-                            } else if (k >= from) {
-                                if (k + 0 < to) y[k] = v.x;
-                                if (k + 1 < to) y[k + 1] = v.y;
-                                if (k + 2 < to) y[k + 2] = v.z;
-                            }
-                        }
+                        for (int j = 0; j < 16; ++j) put4(y, k0 + 2 * j * kStripN, from, to, get(j));
                     }
                 } else {
+                    const unsigned char *Xw = X + 32 * q * 128;
 #pragma unroll 8
                     for (int j = 0; j < kStripN; ++j) {
                         const int rr = j >> 1, k = 32 * j + lane;
@@ -741,7 +1072,12 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
                 }
                 __syncwarp();
             }
-            if (lane == 0) mbar_arrive(&xfree[xs]);
+            if (Sd::MM && !released) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&dfree[ds]);
+            }
+            if (!Sd::MM && lane == 0) mbar_arrive(&xfree[xs]);
             if (q == 0) {
                 trace(i, 12);
                 if (p.trace && lane == 0 && item0 + i < p.trace_tiles) {
@@ -753,6 +1089,7 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
             }
         }
     }
+    if (Sd::MM && P.tma && warp >= 8 && lane == 0) bulk_wait0();  // the outputs are written
     if (Sd::TC) tc_fence_before();
     __syncthreads();
     if (Sd::TC && warp == 1) {
@@ -783,5 +1120,74 @@ __global__ void __launch_bounds__(StripDims<K, TC>::THREADS, 1)
     __syncthreads();
     if (tid == 0) tail->ticket = tail->poison = tail->done = 0;
 }
+
+// ---- launch (one set of instantiations per translation unit: sosfilt_strip_*.cu)
+template <int K, bool NORM, int MODE>
+KernelOnce g_strip_once;
+
+template <int K, bool NORM, int MODE>
+cudaError_t launch_strip_one(const StripParams<K, MODE> &P, cudaStream_t s) {
+    using Sd = StripDims<K, MODE>;
+    auto kern = sos_strip_kernel<K, NORM, MODE>;
+    cudaError_t e = raise_smem_once(g_strip_once<K, NORM, MODE>, kern, Sd::SMEM);
+    if (e != cudaSuccess) return e;
+    kern<<<static_cast<unsigned>(P.cut.n_strips), Sd::THREADS, Sd::SMEM, s>>>(P);
+    return cudaGetLastError();
+}
+
+template <int K, int MODE>
+cudaError_t launch_strip_mode(const LaneParams<K> &p, const StripCut &cut, long long grid, cudaStream_t s) {
+    StripParams<K, MODE> P;
+    std::memset(static_cast<void *>(&P), 0, sizeof(P));
+    P.p = p;
+    P.cut = cut;
+    P.in_place = p.x == p.y;
+    P.x_aligned = reinterpret_cast<uintptr_t>(p.x) % 16 == 0;
+    P.y_aligned = reinterpret_cast<uintptr_t>(p.y) % 16 == 0;
+    P.host_tickets = static_cast<unsigned long long>(p.n_tiles + grid);
+    if constexpr (MODE != kStripFma) {
+        // the tensor maps cost a call about a microsecond on the host: for strips of several units
+        if (P.x_aligned && P.y_aligned && cut.strip_rows >= kStripTmaRows)
+            P.tma = strip_rows_map(&P.tmx, p.x, p.n / kStripN, kStripRows) &&
+                    strip_rows_map(&P.tmy, p.y, p.n / kStripN, 32);
+    }
+    if constexpr (MODE == kStripFma) std::memcpy(P.g, p.gresp, sizeof P.g);
+    return p.norm ? launch_strip_one<K, true, MODE>(P, s) : launch_strip_one<K, false, MODE>(P, s);
+}
+
+template <int K>
+bool launch_strip_k(const LaneParams<K> &p, long long grid, cudaStream_t s, cudaError_t &err) {
+    StripCut cut;
+    if (!p.tail || !p.gimg || !strip_cut(p.n, p.warm_rows, cut)) return false;
+    if constexpr (K > kStripStatesK) {
+        // short signals: the strip kernel's start (operands, products) costs more than a few tiles' lookback
+        // (order 6, 65536 samples: 12.4 us against 10.5; 200000: 12.5 against 12.5; order 16: 14.5 against 16.5
+        // and 15 against 20), the more so where the samples come 4 bytes at a time (order 8, 2.2 M samples: 20.7
+        // against 18.6; 3 M: 20.7 against 22.3)
+        const bool aligned = reinterpret_cast<uintptr_t>(p.x) % 16 == 0;
+        if (cut.n_rows < (aligned || K > 4 ? kStripLeastRows : kStripLeastRows4)) return false;
+    }
+    if constexpr (K <= kStripStatesK) {
+        if (cut.strip_rows + cut.warm_rows <= kStripFmaRows) {
+            err = launch_strip_mode<K, kStripFma>(p, cut, grid, s);
+            return true;
+        }
+    }
+    if constexpr (K > kStripStatesK) {
+        if (p.products) {
+            err = launch_strip_mode<K, kStripOutputs>(p, cut, grid, s);
+            return true;
+        }
+    }
+    err = launch_strip_mode<K, kStripStates>(p, cut, grid, s);
+    return true;
+}
+
+
+#define SOSK_STRIP_INST(k)                                                                           \
+    template <>                                                                                      \
+    bool launch_strip<k>(const LaneParams<k> &p, long long grid, cudaStream_t s, cudaError_t &err) { \
+        return launch_strip_k<k>(p, grid, s, err);                                                   \
+    }
 
 }  // namespace sosk

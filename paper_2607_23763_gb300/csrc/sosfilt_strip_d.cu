@@ -1,0 +1,7 @@
+// The strip kernel (sosfilt_strip.cuh) for section counts 6 (split across translation units so that
+// the build compiles them in parallel).
+#include "sosfilt_strip.cuh"
+
+namespace sosk {
+SOSK_STRIP_INST(6)
+}  // namespace sosk

@@ -2,6 +2,7 @@
 // TMA tensor maps of a launch.
 #include <mutex>
 
+#include "sosfilt_strip.cuh"
 #include "sosfilt_tc.cuh"
 
 namespace sosk {
@@ -30,14 +31,14 @@ EncodeTiledFn encoder() {
     return fn;
 }
 
-// A signal as rows of 64 float32 samples (256-byte row pitch), copied in boxes of 32 x 128 with the
+// A signal as rows of 64 float32 samples (256-byte row pitch), copied in boxes of 32 x box_rows with the
 // 128-byte swizzle the MMA descriptors read; rows past the end load as zeros and are not stored.
-bool encode_rows(CUtensorMap *tm, const float *base, long long rows) {
+bool encode_rows(CUtensorMap *tm, const float *base, long long rows, int box_rows = kTcRows) {
     EncodeTiledFn fn = encoder();
     if (!fn || rows < 1) return false;
     const cuuint64_t dim[2] = {static_cast<cuuint64_t>(kTcN), static_cast<cuuint64_t>(rows)};
     const cuuint64_t stride[1] = {static_cast<cuuint64_t>(kTcN) * sizeof(float)};
-    const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(kTcRows)};
+    const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(box_rows)};
     const cuuint32_t estride[2] = {1, 1};
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dim, stride, box, estride,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -69,6 +70,10 @@ int blocks_k() {
     return blocks_per_sm_once(g_once<K>, sos_tc_kernel<K>, kTcThreads, tc_smem_bytes<K>());
 }
 }  // namespace
+
+bool strip_rows_map(CUtensorMap *tm, const float *base, long long rows, int box_rows) {
+    return encode_rows(tm, base, rows, box_rows);
+}
 
 #define SOSK_TC_INST(k)                                                                                      \
     template <>                                                                                              \

@@ -35,8 +35,9 @@ SIZES = [1, ROW - 1, ROW, ROW + 1, UNIT - 1, UNIT, UNIT + 1, UNIT + UNIT // 2, 3
 
 
 @pytest.mark.parametrize("n", SIZES)
-@pytest.mark.parametrize("order,cutoff", [(2, 0.2), (4, 0.3), (6, 0.1), (10, 0.1), (16, 0.05)])
-def test_sizes_alignment_and_state(dev, order, cutoff, n):
+@pytest.mark.parametrize("order,cutoff,solver", [(2, 0.2, 0), (4, 0.3, 0), (6, 0.1, 0), (6, 0.4, 0), (10, 0.1, 0),
+                                                 (12, 0.4, 0), (16, 0.05, 0), (16, 0.4, 0), (16, 0.4, 4), (14, 0.1, 0)])
+def test_sizes_alignment_and_state(dev, order, cutoff, solver, n):
     """Every size with an initial and a final state, aligned, at odd offsets of input and output, in place
     with the final state over the initial one; all match the oracle, and the in-place result is the
     out-of-place one bit for bit."""
@@ -45,7 +46,7 @@ def test_sizes_alignment_and_state(dev, order, cutoff, n):
     x = workloads.normal_f32(7 + order, n)
     zi = (0.01 * np.random.default_rng(n).standard_normal((K, 2))).astype(np.float32)
     ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
-    f = _filter(sos)
+    f = _filter(sos, tuning={"solver": solver})
     first = None
     for ox, oy in [(0, 0), (1, 2), (3, 0), (0, 1)]:
         xd = torch.empty(n + ox, device=dev)[ox:]
