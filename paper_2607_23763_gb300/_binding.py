@@ -53,6 +53,23 @@ SOLVER_DEFAULT, SOLVER_CR, SOLVER_PH, SOLVER_DTCR, SOLVER_TC = 0, 1, 2, 3, 4
 
 _lib = None
 _lock = threading.Lock()
+_native = None  # native marshalling (csrc/py/native.cpp) where it was built, else False
+_fn = {}        # addresses of the library functions it calls
+
+
+def _native_module():
+    global _native
+    if _native is None:
+        lib = load_library()
+        try:
+            import torch  # noqa: F401  (its libraries are loaded before the module that uses them)
+            from . import _native as mod
+            for name in ("sos_filter_run", "sos_filter_run_noalloc", "sos_filter_run_batch_ex"):
+                _fn[name] = ctypes.cast(getattr(lib, name), ctypes.c_void_p).value
+            _native = mod
+        except ImportError:
+            _native = False
+    return _native
 
 
 def load_library(path: str | None = None):
@@ -146,6 +163,7 @@ class SosFilter:
                                      None if t is None else ctypes.addressof(t), ctypes.byref(h)),
                "sos_filter_create")
         self._h = h
+        self._hv = h.value
         self._lib = lib
 
     @property
@@ -156,6 +174,7 @@ class SosFilter:
         if getattr(self, "_h", None) is not None and self._h.value:
             self._lib.sos_filter_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._hv = 0
 
     def __del__(self):  # pragma: no cover - best effort
         try:
@@ -165,9 +184,15 @@ class SosFilter:
 
     def run(self, x, y=None, zi=None, zf=None, stream=None):
         """y = cascade(x) on the device; x, y, zi, zf are float32 CUDA tensors (y may be x)."""
-        import torch
         if y is None:
+            import torch
             y = torch.empty_like(x)
+        nat = _native if _native is not None else _native_module()
+        if nat:
+            rc = nat.run(_fn["sos_filter_run"], self._hv, x, y, zi, zf, None if stream is None else stream.cuda_stream)
+            if rc:
+                raise SosError(rc, "sos_filter_run")
+            return y
         n = x.numel()
         _check(self._lib.sos_filter_run(self._h, _dptr(x, "x"), _dptr(y, "y"), n,
                                         None if zi is None else _dptr(zi, "zi"),
@@ -180,6 +205,11 @@ class SosFilter:
 
         y must be supplied; at most 2^28 samples per call; calls must not overlap on the GPU.
         """
+        nat = _native if _native is not None else _native_module()
+        if nat:
+            _check(nat.run(_fn["sos_filter_run_noalloc"], self._hv, x, y, zi, zf,
+                           None if stream is None else stream.cuda_stream), "sos_filter_run_noalloc")
+            return y
         _check(self._lib.sos_filter_run_noalloc(self._h, _dptr(x, "x"), _dptr(y, "y"), x.numel(),
                                                 None if zi is None else _dptr(zi, "zi"),
                                                 None if zf is None else _dptr(zf, "zf"), _stream_handle(stream)),
@@ -254,6 +284,14 @@ def run_batch(filters, xs, ys=None, zis=None, zfs=None, stream=None):
     n = len(xs)
     if ys is None:
         ys = [torch.empty_like(x) for x in xs]
+    filters = filters if isinstance(filters, (list, tuple)) else list(filters)
+    zis = zis if zis is None or isinstance(zis, (list, tuple)) else list(zis)
+    zfs = zfs if zfs is None or isinstance(zfs, (list, tuple)) else list(zfs)
+    nat = _native if _native is not None else _native_module()
+    if nat and len(filters) == n and len(ys) == n and (zis is None or len(zis) == n) and (zfs is None or len(zfs) == n):
+        _check(nat.run_batch(_fn["sos_filter_run_batch_ex"], filters, xs, ys, zis, zfs,
+                             None if stream is None else stream.cuda_stream), "sos_filter_run_batch")
+        return ys
     hf = (ctypes.c_void_p * n)(*[f.handle for f in filters])
     hx = (ctypes.c_void_p * n)(*[_dptr(x, "x") for x in xs])
     hy = (ctypes.c_void_p * n)(*[_dptr(y, "y") for y in ys])
