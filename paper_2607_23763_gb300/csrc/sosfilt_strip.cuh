@@ -89,11 +89,16 @@ struct StripDims {
     static constexpr int IMG = MM ? 2 * B1 + 64 * 128 : 4 * kStripImgFloats;
     static constexpr int STAGE = MM ? 4 * WGS * 4096 : 0;
     
+    // from three sections on, the rows' states are formed by two-word products (state_mv2): a warp's four group
+    // states then have every word twice, at a pitch that puts the four on different banks.  Shorter cascades
+    // have too few products to gain by it (order 2, 2^22 samples: 11.9 us against 11.2)
+    static constexpr bool TWO = K > 2;
+    static constexpr int ZW = TWO ? 2 : 1, ZP = !TWO ? S : 2 * S + (S % 8 == 6 ? 8 : 4);
     static constexpr int T_ML = 0;
     static constexpr int T_ACP = T_ML + 11 * Dm::MS;
     static constexpr int T_A = T_ACP + 4 * S * S;
     static constexpr int T_ZV = T_A + WGS * 2 * 4 * S;
-    static constexpr int T_Z = T_ZV + WGS * 4 * 4 * S;
+    static constexpr int T_Z = T_ZV + WGS * 4 * 4 * ZP;
     // the output basis H [S][64] and the states of the signal's first group (row_part), strip 0 only
     static constexpr int T_H = T_Z + kStripZ * S;
     static constexpr int T_ST = T_H + kStripN * S;
@@ -437,6 +442,92 @@ __device__ __forceinline__ float mv_shared(const float *A, const float *x, int r
     return y0 + y1;
 }
 
+// The epilogue's warps fill the issue slots (half of all cycles issue, a fifth of the stalls wait for
+// instructions), so that fewer instructions count for more than shorter chains: order 16, 2^28 samples,
+// 459 -> 421 us by two-word products here, in the scan's coupling and in the operands' remainders (order 12:
+// 375 -> 356, order 8: 375 -> 349; order 16, 2^26 samples: 137 -> 122); a scan that takes the sections in
+// pairs, with half the exchanges in a chain but more products, was slower (473).
+
+// Two float32 in one 64-bit word, and a b + c on both at once.
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// a - b, two words at a time (exact where the difference of each word is) or word by word.
+template <bool TWO>
+__device__ __forceinline__ float4 sub4(const float4 &a, const float4 &b) {
+    if constexpr (!TWO) return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+    const unsigned long long m = pack2(-1.f, -1.f);
+    float4 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(fma2(pack2(b.x, b.y), m, pack2(a.x, a.y))));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.z), "=f"(r.w) : "l"(fma2(pack2(b.z, b.w), m, pack2(a.z, a.w))));
+    return r;
+}
+
+// y += A x, A packed lower block-triangular with its 2 x 2 blocks by columns, x with every word twice, both in
+// shared memory: two-word products, half the instructions.
+template <int K>
+__device__ __forceinline__ void state_mv2(const float *A, const float *x, float (&y)[2 * K]) {
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+        unsigned long long v = pack2(y[2 * s], y[2 * s + 1]);
+#pragma unroll
+        for (int j = 0; j <= s; ++j) {
+            const ulonglong2 B = *reinterpret_cast<const ulonglong2 *>(A + 4 * (s * (s + 1) / 2 + j));
+            const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(x + 4 * j);
+            v = fma2(B.x, z.x, fma2(B.y, z.y, v));
+        }
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(y[2 * s]), "=f"(y[2 * s + 1]) : "l"(v));
+    }
+}
+
+// lane_scan with the sections' coupling in two-word products; p.MX holds the 2 x 2 blocks by columns.
+template <int K, class Secs>
+__device__ __forceinline__ void scan2(const LaneParams<K> &p, const Secs &cs, const float (&t)[2 * K], float (&S)[2 * K],
+                                      float *a_out, int lane) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        unsigned long long v = pack2(t[2 * k], t[2 * k + 1]);
+#pragma unroll
+        for (int j = 0; j < k; ++j) {
+            const float4 b = p.MX[k * (k - 1) / 2 + j];
+            v = fma2(pack2(b.x, b.y), pack2(S[2 * j], S[2 * j]), fma2(pack2(b.z, b.w), pack2(S[2 * j + 1], S[2 * j + 1]), v));
+        }
+        float u1, u2;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(u1), "=f"(u2) : "l"(v));
+#pragma unroll
+        for (int r = 0; r < 5; ++r) {
+            const float o1 = __shfl_up_sync(0xffffffffu, u1, 1 << r);
+            const float o2 = __shfl_up_sync(0xffffffffu, u2, 1 << r);
+            const float4 tn = cs.tn(k, r);
+            if (lane >= (1 << r)) {
+                u1 = fmaf(tn.x, o1, fmaf(tn.y, o2, u1));
+                u2 = fmaf(tn.z, o1, fmaf(tn.w, o2, u2));
+            }
+        }
+        const float s1 = __shfl_up_sync(0xffffffffu, u1, 1), s2 = __shfl_up_sync(0xffffffffu, u2, 1);
+        S[2 * k] = lane == 0 ? 0.f : s1;
+        S[2 * k + 1] = lane == 0 ? 0.f : s2;
+        if (lane == 31) *reinterpret_cast<float2 *>(a_out + 2 * k) = make_float2(u1, u2);
+    }
+}
+
+// Row `lane` (< S) of A x + B y: the two products by a half of the warp each.
+template <int S>
+__device__ __forceinline__ float mv_two(const float *A, const float *x, const float *B, const float *y, int lane) {
+    const bool h = lane >= 16;
+    const float v = mv_shared<S>(h ? B : A, h ? y : x, (lane & 15) < S ? lane & 15 : 0);
+    return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+
 // Words of the run's workspace (LaneParams::tail), all zero between runs.
 struct StripTail {
     unsigned ticket, poison, done, pad;
@@ -536,7 +627,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
         }
         for (int i = k; i < 11 * MS / 4; i += step) {
             const int m = i / (MS / 4), lane_of = m < 8 ? m : 8 * (m - 7);
-            reinterpret_cast<float4 *>(sML)[i] = __ldg(reinterpret_cast<const float4 *>(p.tab) + lane_of * (MS / 4) + i % (MS / 4));
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(p.tab) + lane_of * (MS / 4) + i % (MS / 4));
+            reinterpret_cast<float4 *>(sML)[i] = Sd::TWO ? make_float4(v.x, v.z, v.y, v.w) : v;  // blocks by columns
         }
         for (int i = k; i < 4 * S * S; i += step) sACp[i] = __ldg(p.tab + Dm::OFF_ACP + i);
         if (p.zi && r_first == 0)
@@ -700,8 +792,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     const float4 uh = make_float4(tf32_near(u.x), tf32_near(u.y), tf32_near(u.z), tf32_near(u.w));
                     const float4 vh = make_float4(tf32_near(v.x), tf32_near(v.y), tf32_near(v.z), tf32_near(v.w));
                     tc_st8(t0 + 8 * j, uh, vh);
-                    tc_st8(t0 + 32 + 8 * j, make_float4(u.x - uh.x, u.y - uh.y, u.z - uh.z, u.w - uh.w),
-                           make_float4(v.x - vh.x, v.y - vh.y, v.z - vh.z, v.w - vh.w));
+                    tc_st8(t0 + 32 + 8 * j, sub4<Sd::TWO>(u, uh), sub4<Sd::TWO>(v, vh));
                 }
                 tc_wait_st();
                 tc_fence_before();
@@ -721,7 +812,9 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
         const int r = 32 * q + lane;  // row within the unit
         const unsigned tl = tmem + (static_cast<unsigned>(32 * q) << 16);
         const ParamSecs<K> cs{p};
-        float *zv = tabs + Sd::T_ZV + (wg * 4 + q) * 4 * S;  // [4][S]
+        constexpr int ZP = Sd::ZP, ZW = Sd::ZW;
+        constexpr int QC = Sd::TWO ? 1 : 3;  // the warp that forms the next unit's state
+        float *zv = tabs + Sd::T_ZV + (wg * 4 + q) * 4 * ZP;  // [4][ZP], every word ZW times
         const int li = lane < S ? lane : 0;
         bool dead = false;
         unsigned par = 0, y_par = 0;
@@ -785,7 +878,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     if (lane == 0) mbar_arrive(&dfree[ds]);
                 }
                 if (q == 0) trace(i, 5);
-                lane_scan<K>(cs, t, Sl, ab + q * S, lane);
+                if constexpr (Sd::MM) scan2<K>(p, cs, t, Sl, ab + q * S, lane);
+                else lane_scan<K>(cs, t, Sl, ab + q * S, lane);
                 if (q == 0) trace(i, 7);
             }
             if (!named_bar_and(1 + wg, 128, ok)) break;
@@ -796,17 +890,19 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             float pv = 0.f, cu = 0.f;
             if (q == 1) pv = ab[li];
             if (q == 2) pv = mv_shared<S>(A1, ab, li) + ab[S + li];
-            if (q == 3) {
-                pv = (mv_shared<S>(A2, ab, li) + mv_shared<S>(A1, ab + S, li)) + ab[2 * S + li];
-                cu = (mv_shared<S>(A3, ab, li) + mv_shared<S>(A2, ab + S, li)) +
-                     (mv_shared<S>(A1, ab + 2 * S, li) + ab[3 * S + li]);
+            constexpr bool HALVES = S > 8;  // long rows: two products at a time
+            if (q == 3)
+                pv = (HALVES ? mv_two<S>(A2, ab, A1, ab + S, lane) : mv_shared<S>(A2, ab, li) + mv_shared<S>(A1, ab + S, li)) + ab[2 * S + li];
+            if (q == QC) {
+                cu = (HALVES ? mv_two<S>(A3, ab, A2, ab + S, lane) : mv_shared<S>(A3, ab, li) + mv_shared<S>(A2, ab + S, li)) + ab[3 * S + li];
+                if (!HALVES) cu += mv_shared<S>(A1, ab + 2 * S, li);
             }
             dead = !strip_wait(&zready[i % kStripZ], (i / kStripZ) & 1, budget, p.status);
             if (!Sd::MM && dead) continue;
             if (q == 0) trace(i, 9);
             const float *z0 = z_buf + (i % kStripZ) * S;
-            if (q == 3) {
-                const float zn = mv_shared<S>(A4, z0, li) + cu;
+            if (q == QC) {
+                const float zn = (HALVES ? mv_two<S>(A4, z0, A1, ab + 2 * S, lane) : mv_shared<S>(A4, z0, li)) + cu;
                 if (i + 1 < n_u) {
                     if (lane < S) z_buf[((i + 1) % kStripZ) * S + lane] = zn;
                     __syncwarp();
@@ -822,7 +918,10 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 const float zq = q == 0 ? z0[li] : mv_shared<S>(q == 1 ? A1 : q == 2 ? A2 : A3, z0, li) + pv;
                 // (M_N)^lane Z_v in two steps, lane = 8 a + b: the four (M_N)^(8 a) Z_v, a section's two words a
                 // lane, then each lane's (M_N)^b of one of them (11 matrices to read instead of 32)
-                if (lane < S) zv[lane] = zq;
+                if (lane < S) {
+                    if constexpr (Sd::TWO) *reinterpret_cast<float2 *>(zv + 2 * lane) = make_float2(zq, zq);
+                    else zv[lane] = zq;
+                }
                 __syncwarp();
                 {
                     const int a = lane >> 3, s = lane & 7;
@@ -833,18 +932,20 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                         for (int j = 0; j < K; ++j)
                             if (j <= s) {
                                 const float4 B = *reinterpret_cast<const float4 *>(m + 4 * j);
-                                const float2 z = *reinterpret_cast<const float2 *>(zv + 2 * j);
-                                w0 = fmaf(B.x, z.x, fmaf(B.y, z.y, w0));
-                                w1 = fmaf(B.z, z.x, fmaf(B.w, z.y, w1));
+                                const float z0 = zv[2 * ZW * j], z1 = zv[2 * ZW * j + ZW];
+                                w0 = fmaf(B.x, z0, fmaf(Sd::TWO ? B.z : B.y, z1, w0));
+                                w1 = fmaf(Sd::TWO ? B.y : B.z, z0, fmaf(B.w, z1, w1));
                             }
-                        *reinterpret_cast<float2 *>(zv + a * S + 2 * s) = make_float2(w0, w1);
+                        if constexpr (Sd::TWO) *reinterpret_cast<float4 *>(zv + a * ZP + 4 * s) = make_float4(w0, w0, w1, w1);
+                        else *reinterpret_cast<float2 *>(zv + a * ZP + 2 * s) = make_float2(w0, w1);
                     }
                 }
                 __syncwarp();
                 float st[S];
 #pragma unroll
                 for (int j = 0; j < S; ++j) st[j] = Sl[j];
-                lane_state_mv<K>(sML + (lane & 7) * MS, zv + (lane >> 3) * S, st);
+                if constexpr (Sd::TWO) state_mv2<K>(sML + (lane & 7) * MS, zv + (lane >> 3) * ZP, st);
+                else lane_state_mv<K>(sML + (lane & 7) * MS, zv + (lane >> 3) * ZP, st);
                 unsigned char *X = sm + xs * kStripXBytes;
                 const long long base = R * kStripN;
                 if (q == 0) trace(i, 10);
@@ -920,7 +1021,12 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     for (int j = 0; j < 16; ++j) e[j] = j < S ? tf32_near(st[j < S ? j : 0]) : 0.f;
                     tc_st16(tl + ds * Sd::COLS + 64, e);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) e[j] = j < S ? st[j < S ? j : 0] - e[j] : 0.f;
+                    for (int j = 0; j < 16; j += 4) {
+                        const float4 l = sub4<true>(make_float4(j < S ? st[j < S ? j : 0] : 0.f, j + 1 < S ? st[j + 1 < S ? j + 1 : 0] : 0.f,
+                                                          j + 2 < S ? st[j + 2 < S ? j + 2 : 0] : 0.f, j + 3 < S ? st[j + 3 < S ? j + 3 : 0] : 0.f),
+                                              make_float4(e[j], e[j + 1], e[j + 2], e[j + 3]));
+                        e[j] = l.x; e[j + 1] = l.y; e[j + 2] = l.z; e[j + 3] = l.w;
+                    }
                     tc_st16(tl + ds * Sd::COLS + 80, e);
                     tc_wait_st();
                     tc_fence_before();
@@ -1140,6 +1246,8 @@ cudaError_t launch_strip_mode(const LaneParams<K> &p, const StripCut &cut, long 
     StripParams<K, MODE> P;
     std::memset(static_cast<void *>(&P), 0, sizeof(P));
     P.p = p;
+    if constexpr (MODE == kStripOutputs)
+        for (auto &b : P.p.MX) b = make_float4(b.x, b.z, b.y, b.w);  // by columns (scan2)
     P.cut = cut;
     P.in_place = p.x == p.y;
     P.x_aligned = reinterpret_cast<uintptr_t>(p.x) % 16 == 0;
