@@ -97,9 +97,10 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
     // only its own capture, after its own correction has read it (another warp may run two tiles
     // ahead, into the same slot, before this one corrects)
     float *zs_tail = agg + 2 * S;
+    BatchSig *ring_sig = reinterpret_cast<BatchSig *>(zs_tail + 2 * W * SZ);  // [8] the tickets' signals
+    static_assert(sizeof(BatchSig) == 96 && (RSP % 2) == 0, "descriptors are copied as 64-bit words");
     __shared__ unsigned long long bar_local[2], bar_zready[2], bar_ticket[8];
     __shared__ long long ring[8];
-    __shared__ int ring_sig[8];
     __shared__ int fold_count[2];
     __shared__ int tickets_exhausted;
 
@@ -107,22 +108,36 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
     const int warp = threadIdx.x >> 5;
     const long long budget = p.spin_budget;
 
-    // Tickets: tile of iteration k in ring[k & 7] with its signal in ring_sig[k & 7], posted on
-    // bar_ticket[k & 7] (phase (k >> 3) & 1).  Thread 0 draws the first two; afterwards the folding
+    // Tickets: tile of iteration k in ring[k & 7] with its signal's descriptor in ring_sig[k & 7], posted on
+    // bar_ticket[k & 7] (phase (k >> 3) & 1).  The first warp draws the first two; afterwards the folding
     // warp of iteration k draws k + 2 (two ahead, not three: tiles are then numbered closer to when
     // blocks reach them, and a tile's predecessors fold closer to it -- 6 % faster on the batched
-    // mix), which still leaves a tile's input staged one iteration ahead.
+    // mix), which still leaves a tile's input staged one iteration ahead.  The descriptor comes with
+    // the ticket, so that no warp waits on global memory for it before its loads, its recurrences or
+    // its stores, and the draw follows the tile's hand-over to the coordinator, which it held up by
+    // three dependent global accesses: 192 signals of orders 2 to 16 (88 M samples) 333 -> 325 us, 24
+    // signals of 4 M samples 608 -> 583 us at order 16, 353 -> 341 at 8, 254 -> 246 at 4, 226 -> 220 at 2.
+    // Called by a whole warp.
     auto draw_ticket = [&](int slot) {
         long long t = -1;
-        if (!tickets_exhausted) {
-            t = static_cast<long long>(atomicAdd(p.ticket, 1ULL) - p.ticket_base);
-            if (t >= p.n_tiles) {
-                tickets_exhausted = 1;
-                t = -1;
+        int sig = -1;
+        if (lane == 0) {
+            if (!tickets_exhausted) {
+                t = static_cast<long long>(atomicAdd(p.ticket, 1ULL) - p.ticket_base);
+                if (t >= p.n_tiles) {
+                    tickets_exhausted = 1;
+                    t = -1;
+                }
             }
+            ring[slot] = t;
+            if (t >= 0) sig = __ldg(p.tile_sig + t);
         }
-        ring[slot] = t;
-        ring_sig[slot] = t >= 0 ? __ldg(p.tile_sig + t) : -1;
+        sig = __shfl_sync(0xffffffffu, sig, 0);
+        if (sig >= 0 && lane < static_cast<int>(sizeof(BatchSig) / 8))
+            reinterpret_cast<unsigned long long *>(&ring_sig[slot])[lane] =
+                __ldg(reinterpret_cast<const unsigned long long *>(p.sigs + sig) + lane);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_ticket[slot]);
     };
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -133,11 +148,10 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
         tickets_exhausted = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) mbar_init(&bar_ticket[i], 1);
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            draw_ticket(i);
-            mbar_arrive(&bar_ticket[i]);
-        }
+    }
+    if (warp == 0) {
+        __syncwarp();
+        for (int i = 0; i < 2; ++i) draw_ticket(i);
     }
     __syncthreads();
 
@@ -150,7 +164,7 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
             if (!mbar_wait(&bar_ticket[it & 7], (it >> 3) & 1, budget, p.status)) break;
             const long long cur = ring[it & 7];
             if (cur < 0) break;
-            const BatchSig *sg = p.sigs + ring_sig[it & 7];
+            const BatchSig *sg = &ring_sig[it & 7];
             const long long tile0 = sg->tile0;
             const float *tab = sg->tab;
             const float *zi = sg->zi;
@@ -266,13 +280,13 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
         cp_async_commit();
     };
 
-    // Correction of the tile of iteration jt (signal sig), whose particular output is in buffer Y
+    // Correction of the tile of iteration jt, whose particular output is in buffer Y
     // and whose lanes' scan states are Sl: rows' true states to shared memory, then four samples per
     // lane across the rows, stored straight to y.
-    auto correct_and_store = [&](long long tile, int sig, unsigned jt, const float *Y, const float (&Sl)[S]) -> bool {
+    auto correct_and_store = [&](long long tile, unsigned jt, const float *Y, const float (&Sl)[S]) -> bool {
         const unsigned slot = jt & 1;
         if (!mbar_wait(&bar_zready[slot], (jt >> 1) & 1, budget, p.status)) return false;
-        const BatchSig *sg = p.sigs + sig;
+        const BatchSig *sg = &ring_sig[jt & 7];
         const long long g = (tile - sg->tile0) * W + w;
         const long long G = sg->G;
         float st[S];
@@ -340,12 +354,10 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
 
     if (!mbar_wait(&bar_ticket[0], 0, budget, p.status)) return;
     long long tile = ring[0];
-    int sig = ring_sig[0];
     if (tile < 0) return;
-    issue_load(tile, p.sigs + sig, B0);
+    issue_load(tile, &ring_sig[0], B0);
     unsigned it = 0;
     long long prev = -1;
-    int prev_sig = -1;
     float Sprev[S];
 #pragma unroll
     for (int j = 0; j < S; ++j) Sprev[j] = 0.f;
@@ -353,7 +365,7 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
     int cur_buf = 0;  // buffer of this iteration's tile; the next tile goes to (cur_buf + 1) % 3
     for (;;) {
         const unsigned slot = it & 1;
-        const BatchSig *sg = p.sigs + sig;
+        const BatchSig *sg = &ring_sig[it & 7];
         const long long g = (tile - sg->tile0) * W + w;
         const long long G = sg->G;
         float *X = B0 + cur_buf * kL * P;
@@ -366,8 +378,7 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
             break;
         }
         const long long next = ring[(it + 1) & 7];
-        const int next_sig = ring_sig[(it + 1) & 7];
-        if (next >= 0) issue_load(next, p.sigs + next_sig, B0 + nxt_buf * kL * P);
+        if (next >= 0) issue_load(next, &ring_sig[(it + 1) & 7], B0 + nxt_buf * kL * P);
 
         float t[S], Sl[S];
         if (g < G) {
@@ -408,30 +419,25 @@ __device__ __forceinline__ void batch_body(const BatchParams<K> &p, float4 *smem
                 if (tile > sg->tile0 && lane < S)
                     st_relaxed_b64(p.desc + static_cast<size_t>(tile) * 2 * S + lane, pack_word((p.epoch << 2) | 1u, c));
                 if (lane < S) agg[slot * S + lane] = c;
-                if (lane == 0) {
-                    fold_count[slot] = 0;
-                    draw_ticket((it + 2) & 7);
-                    mbar_arrive(&bar_ticket[(it + 2) & 7]);
-                }
+                if (lane == 0) fold_count[slot] = 0;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bar_local[slot]);
+                draw_ticket((it + 2) & 7);
             }
         }
-        if (prev >= 0 && !correct_and_store(prev, prev_sig, it - 1, B0 + prv_buf * kL * P, Sprev)) {
+        if (prev >= 0 && !correct_and_store(prev, it - 1, B0 + prv_buf * kL * P, Sprev)) {
             ok = false;
             break;
         }
 #pragma unroll
         for (int j = 0; j < S; ++j) Sprev[j] = Sl[j];
         prev = tile;
-        prev_sig = sig;
         if (next < 0) break;
         tile = next;
-        sig = next_sig;
         cur_buf = nxt_buf;
         ++it;
     }
-    if (ok) correct_and_store(prev, prev_sig, it, B0 + cur_buf * kL * P, Sprev);
+    if (ok) correct_and_store(prev, it, B0 + cur_buf * kL * P, Sprev);
     cp_async_wait_all();
 }
 
@@ -447,7 +453,7 @@ template <int K, int N>
 constexpr size_t batch_smem_bytes() {
     using Dm = LaneDims<K, N, kBatchW>;
     return sizeof(float) * (static_cast<size_t>(kBatchW) * 3 * kL * (N + 4) + kBatchW * kL * Dm::RSP +
-                            4 * kBatchW * Dm::S + 2 * Dm::S + 2 * kBatchW * ((Dm::S + 3) / 4) * 4);
+                            4 * kBatchW * Dm::S + 2 * Dm::S + 2 * kBatchW * ((Dm::S + 3) / 4) * 4) + 8 * sizeof(BatchSig);
 }
 
 }  // namespace sosk
