@@ -167,6 +167,15 @@ constexpr int kStripTmaRows = 4 * kStripRows;
 // A signal's full rows of 64 samples as a tensor map, copied in boxes of 32 x box_rows (sosfilt_tc.cu).
 bool strip_rows_map(CUtensorMap *tm, const float *base, long long rows, int box_rows);
 
+// The recurrences' coefficients of the sections s and s + H, H = K / 2, in one word each (lane_recurrence): -a1,
+// -a2, and of the sections after them b1, b2, b0 (zero past the last).
+template <int K>
+struct StripPairs {
+    static constexpr bool TWO = K > 2 && K % 2 == 0;
+    static constexpr int H = (K + 1) / 2;
+    unsigned long long a1[H], a2[H], b1[H], b2[H], b0[H];
+};
+
 template <int K, int MODE>
 struct StripParams {
     LaneParams<K> p;
@@ -176,6 +185,7 @@ struct StripParams {
     int tma;           // tmx and tmy are set: full units are loaded, full groups' outputs stored by TMA
     CUtensorMap tmx, tmy;  // x and y as [rows][64], boxes of 32 x 128 and 32 x 32, 128-byte swizzle
     unsigned long long host_tickets;  // what the host adds to the lookback kernels' ticket base
+    StripPairs<K> pk;
     float g[MODE == kStripFma ? 2 * K : 1][kStripN];  // without the tensor cores: the state responses
 };
 
@@ -246,6 +256,23 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
     return v;
 }
 
+// Two float32 in one 64-bit word, and a b + c on both at once.
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ void unpack2(unsigned long long v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+
 // The sections' recurrences over one row (64 samples, in place) from the row's true incoming state st
 // (transposed direct form II), sections skewed by one sample each and in direct-form-I order as in
 // lane_particular: a state word z1, z2 enters its section's input at the section's samples 0 and 1.
@@ -254,9 +281,16 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
 // the loads and stores with the dependent FMAs of a step (one section, one warp per scheduler: 1000 cycles
 // a row instead of 2800); with U = 1 the code stays small where every scheduler has work (unrolling by 2 to
 // 8 cost 7 to 17 % at orders 2 to 16 on 2^26 samples and more, in instruction fetches).
+//
+// Four, six and eight sections (TWO): the steps take sections s and s + H, H = K / 2, in one two-word product
+// each, with the coefficients from `pk` (StripPairs): the inputs of the pair s are the outputs of the pair
+// s - 1 as they lie, and only the pair 0 puts two words together.  The same products in the same order, in half
+// the issue slots, which is what bounds the recurrences here: 2^28 samples, order 8 486 -> 460 us, order 12
+// 605 -> 586, order 16 751 -> 677.  An odd count wastes half a pair (orders 6 and 10 were 3 and 7 % slower
+// so); two sections are one pair that waits on itself.
 template <int K, bool NORM, int U, class Secs>
-__device__ __forceinline__ void lane_recurrence(const Secs &cs, unsigned char *sm, unsigned row, float gain,
-                                                const float (&st)[2 * K]) {
+__device__ __forceinline__ void lane_recurrence(const Secs &cs, const StripPairs<K> &pk, unsigned char *sm, unsigned row,
+                                                float gain, const float (&st)[2 * K]) {
     constexpr int N = kStripN, D = K - 1, R0 = (4 - (D & 3)) & 3, D4 = (D + R0) / 4;
     constexpr int C0 = ((K + 1 + 3) / 4 + U - 1) / U * U;  // chunks in which some section starts: unrolled
     float y1[K], y2[K], pipe[K];
@@ -341,6 +375,57 @@ __device__ __forceinline__ void lane_recurrence(const Secs &cs, unsigned char *s
         if (j + 1 < N / 4) xn = get(at_chunk(j + 1));
         chunk(at_chunk(j), xv, 4 * j);
     }
+    if constexpr (StripPairs<K>::TWO) {
+        using W = unsigned long long;
+        constexpr int H = StripPairs<K>::H, LAST = H - 1;  // the pair whose second section is the last
+        static_assert(U == 1);
+        W Y1[H], Y2[H], PP[H];
+#pragma unroll
+        for (int s = 0; s < H; ++s) {
+            Y1[s] = pack2(y1[s], y1[s + H]);
+            Y2[s] = pack2(y2[s], y2[s + H]);
+            PP[s] = pack2(pipe[s], pipe[s + H]);
+        }
+#pragma unroll 1
+        for (int j0 = C0; j0 < N / 4; ++j0) {
+            const float4 xv = xn;
+            if (j0 + 1 < N / 4) xn = get(at_chunk(j0 + 1));
+#pragma unroll
+            for (int r = D4; r > 0; --r) at[r] = at[r - 1];
+            at[0] = at_chunk(j0);
+            const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+            float out[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float mid, over;  // the input of section H: what section H - 1 left in the last step
+                unpack2(PP[H - 1], mid, over);
+                const float F0 = input(xs[j]);
+#pragma unroll
+                for (int s = H - 1; s >= 0; --s) {
+                    const W F = s > 0 ? PP[s > 0 ? s - 1 : 0] : pack2(F0, mid);
+                    const W y = fma2(pk.a1[s], Y1[s], fma2(pk.a2[s], Y2[s], F));
+                    W by = y;
+                    if constexpr (!NORM) asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(by) : "l"(pk.b0[s]), "l"(y));
+                    PP[s] = fma2(pk.b1[s], Y1[s], fma2(pk.b2[s], Y2[s], by));
+                    Y2[s] = Y1[s];
+                    Y1[s] = y;
+                    if (s == LAST) unpack2(y, over, out[j]);
+                }
+            }
+            float blk[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) blk[r] = r < R0 ? carry[r] : out[r - R0];
+            *reinterpret_cast<float4 *>(sm + at[D4]) = make_float4(blk[0], blk[1], blk[2], blk[3]);
+#pragma unroll
+            for (int r = 0; r < R0; ++r) carry[r] = out[4 - R0 + r];
+        }
+#pragma unroll
+        for (int s = 0; s < H; ++s) {
+            unpack2(Y1[s], y1[s], y1[s + H]);
+            unpack2(Y2[s], y2[s], y2[s + H]);
+            unpack2(PP[s], pipe[s], pipe[s + H]);
+        }
+    } else {
 #pragma unroll 1
     for (int j0 = C0; j0 < N / 4; j0 += U) {
         const unsigned b = at_chunk(j0);
@@ -353,6 +438,7 @@ __device__ __forceinline__ void lane_recurrence(const Secs &cs, unsigned char *s
                 xn = get(at_chunk(j0 + U));
             chunk(b ^ (u << 4), xv, 4 * C0);
         }
+    }
     }
     // drain: steps N .. N + D - 1, in which only the sections s > step - N are still running
     if constexpr (D > 0) {
@@ -447,19 +533,6 @@ __device__ __forceinline__ float mv_shared(const float *A, const float *x, int r
 // 459 -> 421 us by two-word products here, in the scan's coupling and in the operands' remainders (order 12:
 // 375 -> 356, order 8: 375 -> 349; order 16, 2^26 samples: 137 -> 122); a scan that takes the sections in
 // pairs, with half the exchanges in a chain but more products, was slower (473).
-
-// Two float32 in one 64-bit word, and a b + c on both at once.
-__device__ __forceinline__ unsigned long long pack2(float a, float b) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 // a - b, two words at a time (exact where the difference of each word is) or word by word.
 template <bool TWO>
@@ -1057,7 +1130,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                             st[j] = 0.f;
                         }
                     }
-                    lane_recurrence<K, NORM, Sd::U>(cs, sm, row, p.gain, st);
+                    lane_recurrence<K, NORM, Sd::U>(cs, P.pk, sm, row, p.gain, st);
                     if (first) row_part<K>(sm, row, tabs + Sd::T_H, tabs + Sd::T_ST + lane * S);
                     __syncwarp();
                 }
@@ -1260,6 +1333,19 @@ cudaError_t launch_strip_mode(const LaneParams<K> &p, const StripCut &cut, long 
                     strip_rows_map(&P.tmy, p.y, p.n / kStripN, 32);
     }
     if constexpr (MODE == kStripFma) std::memcpy(P.g, p.gresp, sizeof P.g);
+    if constexpr (MODE == kStripStates && StripPairs<K>::TWO) {
+        constexpr int H = StripPairs<K>::H;
+        auto put = [](unsigned long long &w, int half, float v) { std::memcpy(reinterpret_cast<char *>(&w) + 4 * half, &v, 4); };
+        for (int k = 0; k < K; ++k) {
+            const int s = k % H, half = k / H;
+            put(P.pk.a1[s], half, p.sec[k].c.z);
+            put(P.pk.a2[s], half, p.sec[k].c.w);
+            if (k + 1 == K) continue;
+            put(P.pk.b1[s], half, p.sec[k + 1].c.x);
+            put(P.pk.b2[s], half, p.sec[k + 1].c.y);
+            put(P.pk.b0[s], half, p.sec[k + 1].b0);
+        }
+    }
     return p.norm ? launch_strip_one<K, true, MODE>(P, s) : launch_strip_one<K, false, MODE>(P, s);
 }
 

@@ -86,6 +86,28 @@ def test_matches_the_lookback_kernel(dev, order, n):
     b.close()
 
 
+@pytest.mark.parametrize("n", [2048 * ROW, (1 << 20) + 77, 3 * SMS * UNIT + ROW - 1])
+@pytest.mark.parametrize("zero_b0", [False, True])
+@pytest.mark.parametrize("order", [6, 8, 10, 12, 16])
+def test_recurrences_of_a_quiet_cascade(dev, order, zero_b0, n):
+    """Cascades of little float32 noise (below 5e-7 of the output) are done by the recurrences, even counts of
+    sections two at a time, with every section's b0 factored out and with a b0 of zero (the general class).
+    Bound: ten times that noise."""
+    sos = designs.butter_lowpass(order, 0.5)
+    if zero_b0:
+        sos[1] = [0.0, 1.0, 0.5, sos[1, 3], sos[1, 4]]
+    x = workloads.normal_f32(order, n)
+    zi = (0.01 * np.random.default_rng(n).standard_normal((order // 2, 2))).astype(np.float32)
+    ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
+    f = _filter(sos)
+    zf = torch.empty(order // 2, 2, device=dev)
+    y = f.run(torch.from_numpy(x).to(dev), zi=torch.from_numpy(zi).to(dev), zf=zf)
+    assert f.sync_status() == 0
+    assert oracle.rel_err(y.cpu().numpy(), ref) < 5e-6
+    assert np.abs(zf.cpu().numpy() - zref).max() < 5e-6 * max(np.abs(zref).max(), np.abs(ref).max())
+    f.close()
+
+
 @pytest.mark.parametrize("radius", [0.9, 0.999, 0.99999])
 def test_long_memory(dev, radius):
     """Cascades that remember for a part of a strip, for several units, and for longer than a strip (those
