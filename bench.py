@@ -42,18 +42,28 @@ CPU_SAMPLE = 1 << 24  # oracle sample per step of the reference arm
 # removed) whenever its kernel changes.
 SOLVER_CR, SOLVER_PH, SOLVER_DTCR, SOLVER_TC = 1, 2, 3, 4
 TRAFFIC_BYTES_2P28 = {
-    # sos_lane_kernel<8, 64, 7> at 2^26 samples: 268,859,904 B read + 211,708,672 B written
-    (SOLVER_PH, 64): 4 * (268859904 + 211708672),
-    # sos_tc_kernel<8> at 2^26 samples: 269,061,632 B read + 213,409,792 B written
-    (SOLVER_TC, 64): 4 * (269061632 + 213409792),
+    # sos_strip_kernel<8> (both PH solvers) at 2^26 samples: 275,840,000 B read + 214,487,552 B written
+    (SOLVER_PH, 64): 4 * (275840000 + 214487552),
+    (SOLVER_TC, 64): 4 * (275840000 + 214487552),
 }
 PH_GROUPS_PER_BLOCK = 7
 CR_GROUPS_PER_BLOCK = {32: 8, 64: 4}
 
 
+def runs_by_strips(solver: int, N: int, W: int = 0) -> bool:
+    """Whether a long run of this benchmark's Butterworth filters (stable, forgetting their state within a few
+    thousand samples) is taken strip by strip: both PH solvers at N = 64 and 7 or 8 groups per tile."""
+    return solver in (SOLVER_PH, SOLVER_TC) and N == 64 and W in (0, 7, 8)
+
+
 def kernel_name(solver: int, N: int, K: int, W: int = 0) -> str:
     """The kernel a run launches, by solver, samples per lane, sections per pass and groups per tile."""
     k = min(K, 8)
+    if runs_by_strips(solver, N, W):
+        how = ("terminal states by tcgen05 TF32 products, outputs by recurrences" if k <= 2 else
+               "outputs and terminal states by tcgen05 TF32 products split three ways, TMA staging")
+        return (f"sos_strip_kernel<{k}> (PH factorization by strips without lookback: {how}; {k} sections, "
+                "N = 64 samples per lane, units of 128 rows, one strip per SM)")
     if solver == SOLVER_PH:
         w = W or PH_GROUPS_PER_BLOCK
         return (f"sos_lane_kernel<{k}, {N}, {w}> (PH factorization, {k} sections, N = {N} samples per lane, "
@@ -280,12 +290,13 @@ def fp32_fma_roof(torch, dev, sm_max_mhz):
 
 
 def tc_tensor_roofline(K: int, n: int, ms: float) -> dict:
-    """Tensor-core roofline of the PH kernel on the tensor cores.  Per 128-row unit (8192 samples) it
-    issues 24 TF32 MMAs of 128 x 80 x 8 (the Toeplitz and state-response products, three ways) and 6
-    (2K <= 8: 3) of 128 x 64 x 8 (the correction), i.e. 576 (528) flops per sample; the peak is the
-    measured bf16 burst rate times the nominal TF32 / bf16 ratio 1.1 / 2.25."""
+    """Tensor-core roofline of the strip kernel at three and more sections.  Per 128-row unit (8192 samples) it
+    issues three chains (the splits) of eight TF32 MMAs of 128 x (80, 80, 64, 64, 48, 48, 32, 32) x 8 -- the
+    columns of the Toeplitz and state-response image that are not zero -- and 6 (2K <= 8: 3) of 128 x 64 x 8
+    (the correction), i.e. 432 (384) flops per sample; the peak is the measured bf16 burst rate times the
+    nominal TF32 / bf16 ratio 1.1 / 2.25."""
     corr = 6 if K > 4 else 3
-    flops_per_sample = (24 * 2 * 128 * 80 * 8 + corr * 2 * 128 * 64 * 8) / 8192
+    flops_per_sample = (3 * 448 * 2 * 128 * 8 + corr * 2 * 128 * 64 * 8) / 8192
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
             bf16, kind = float(json.load(fh)["bf16_tflops"]), "measured"
@@ -548,7 +559,8 @@ def bench_ours(args):
     clocks = clk.summary()
     # the FP32 roof the method meets first at high order: its FMAs per sample (PH: 4K for the
     # particular pass with b0 = 1 plus 2K for the correction; cyclic reduction: 8K + 2K, Sec. IV-C)
-    fma_per_sample = 6 * K if kid[0] == SOLVER_PH else 10 * K
+    # (the strip kernel's recurrences: 4K, from the row's true state)
+    fma_per_sample = 4 * K if runs_by_strips(*kid) else 6 * K if kid[0] == SOLVER_PH else 10 * K
     fma_peak, fma_kind = fp32_fma_roof(torch, dev, clocks.get("sm_max_mhz"))
     alu_achieved = fma_per_sample * N_SAMPLES / (ms_step * 1e-3) / 1e12
     traffic = (TRAFFIC_BYTES_2P28.get(kid[:2]) if (N_SAMPLES == 1 << 28 and ORDER == 16 and not args.lbw
@@ -573,7 +585,7 @@ def bench_ours(args):
         "gpu_launches": args.steps,
         "clocks": clocks,
     }
-    if kid[0] == SOLVER_TC:
+    if runs_by_strips(*kid) and K > 2:
         # the products run on the tensor cores, not the FP32 pipe: their TF32 rate instead
         line.pop("roofline_alu")
         line["roofline_tensor"] = tc_tensor_roofline(K, N_SAMPLES, ms_step)

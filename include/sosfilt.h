@@ -12,7 +12,9 @@
  * states are carried across groups by decoupled lookback (Sec. IV-B, Eq. 25) and
  * the homogeneous correction (Eq. 24) is applied once a group's incoming state
  * is known.  All K sections of a group stay in registers inside one kernel
- * (Sec. IV-A).
+ * (Sec. IV-A).  Runs by the PH solvers at N = 64 of a cascade that forgets its state
+ * within a strip of the signal need no lookback: every SM filters one contiguous strip,
+ * started early from zero state by the samples after which a state has vanished in float32.
  *
  * Conventions used by every entry point
  *   - Coefficients: `sos` is a host array [n_sections][5] of double holding
@@ -90,7 +92,9 @@ enum {
                                lanes' true states with the output basis; TF32 products with every
                                float32 operand split into head and remainder (float32 accuracy).
                                Cascade carry only, N = 64, tiles of 8 groups.  Needs x and y
-                               16-byte aligned and n >= 64; other runs use SOS_SOLVER_PH */
+                               16-byte aligned and n >= 64; other runs use SOS_SOLVER_PH.
+                               By strips (below) both solvers use the tensor cores, SOS_SOLVER_PH
+                               for the outputs too where its float32 rounding is no smaller */
 };
 
 /*
@@ -107,7 +111,7 @@ enum {
  *                      to stay within 168 registers); any other solver: 0
  *   threads_per_group  L (one thread group per signal block group, Sec. IV-D)
  *   fp64_carry         reserved: must be 0 (carries are float32)
- *   spin_budget_cycles upper bound, in SM clock cycles, on one lookback wait;
+ *   spin_budget_cycles upper bound, in SM clock cycles, on one lookback or barrier wait;
  *                      on expiry the kernel records SOS_ETIMEOUT and returns
  *   lookback_width     per-section carries only: predecessors read per lookback
  *                      round, in units of 32: 1, 2, 4, 8 or 16 (values other than
@@ -125,7 +129,8 @@ enum {
  *                      IV-B) and may differ in the last ulps; 1 requests reproducible results and
  *                      is rejected with SOS_EINVAL together with solver SOS_SOLVER_CR or
  *                      SOS_SOLVER_DTCR, a carry other than SOS_CARRY_DEFAULT, a lookback width or
- *                      N = 128.
+ *                      N = 128.  Runs by strips sum nothing across blocks and repeat bit for
+ *                      bit as well on the same device model.
  */
 typedef struct {
     int N, L, groups_per_cta, threads_per_group, fp64_carry;
@@ -165,7 +170,7 @@ sos_status sos_filter_destroy(sos_filter *f);
  *   zf_dev  device float32[K][2] receives the final state, or NULL; may equal zi_dev
  *   stream  cudaStream_t as void*
  * Ownership: the caller owns x, y, zi, zf; the library owns its workspace
- * (lookback descriptors, ticket counter, status word), grown on demand.
+ * (lookback descriptors, ticket counter, strips' words, status word), grown on demand.
  * CUDA graphs: a run may be captured into a graph on `stream` (solvers PH, DTCR and
  * cyclic reduction with the cascade carry; per-section carries give SOS_EINVAL).
  * A captured run resets its own ticket counter and lookback descriptors inside the
