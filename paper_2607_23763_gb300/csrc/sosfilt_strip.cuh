@@ -869,6 +869,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 }
                 tc_wait_st();
                 tc_fence_before();
+                // the unit's samples have been read, by ordinary loads, before a TMA copy overwrites the stage
+                if (P.tma && h == 1) fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&afull[h]);
             }
@@ -1256,7 +1258,13 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&dfree[ds]);
             }
-            if (!Sd::MM && lane == 0) mbar_arrive(&xfree[xs]);
+            if (!Sd::MM) {
+                // the recurrences' ordinary stores to the stage, and the loads of the outputs, come before the TMA
+                // copy that overwrites it
+                if (Sd::TC && P.tma) fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&xfree[xs]);
+            }
             if (q == 0) {
                 trace(i, 12);
                 if (p.trace && lane == 0 && item0 + i < p.trace_tiles) {

@@ -171,3 +171,60 @@ def test_streams_and_filters_at_once(dev):
     assert all(f.sync_status() == 0 for f in fs)
     for f in fs:
         f.close()
+
+
+def _five_units_a_strip(dev):
+    """Samples of a signal whose strips are long enough (512 rows and more) for TMA copies."""
+    return 5 * torch.cuda.get_device_properties(dev).multi_processor_count * UNIT
+
+
+# what forms the outputs: recurrences of one and two sections, in pairs, one at a time; products (both solvers)
+LONG = [(2, 0.2, 0), (4, 0.3, 0), (8, 0.5, 0), (12, 0.5, 0), (6, 0.5, 0), (16, 0.05, 0), (8, 0.1, 0), (16, 0.4, 4)]
+
+
+@pytest.mark.parametrize("tail", [0, 77])
+@pytest.mark.parametrize("order,cutoff,solver", LONG)
+def test_strips_by_tma(dev, order, cutoff, solver, tail):
+    """Strips long enough for TMA copies, with an initial and a final state: against the oracle, and the run in
+    place, with the final state over the initial one, bit for bit the same."""
+    sos = designs.butter_lowpass(order, cutoff)
+    n = _five_units_a_strip(dev) + tail
+    x = workloads.normal_f32(11 + order, n)
+    zi = (0.01 * np.random.default_rng(order).standard_normal((order // 2, 2))).astype(np.float32)
+    ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
+    f = _filter(sos, tuning={"solver": solver})
+    xd, z, zf = torch.from_numpy(x).to(dev), torch.from_numpy(zi).to(dev), torch.empty(order // 2, 2, device=dev)
+    y = torch.full((n + 8,), 7.0, device=dev)
+    f.run(xd, y[:n], zi=z, zf=zf)
+    assert f.sync_status() == 0
+    assert bool((y[n:] == 7.0).all())
+    assert oracle.rel_err(y[:n].cpu().numpy(), ref) < 1e-4
+    assert np.abs(zf.cpu().numpy() - zref).max() < 1e-4 * np.abs(zref).max()
+    f.run(xd, xd, zi=z, zf=z)
+    assert f.sync_status() == 0
+    assert torch.equal(xd, y[:n]) and torch.equal(z, zf)
+    f.close()
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("bad", [float("nan"), float("-inf")])
+@pytest.mark.parametrize("order,cutoff", [(2, 0.2), (8, 0.5), (16, 0.05)])
+@pytest.mark.parametrize("long", [False, True])
+def test_values_that_are_not_finite_in_every_mode(dev, order, cutoff, bad, in_place, long):
+    """The same for each way of forming the outputs (order 16 at 0.05: products, whose rows with such samples are
+    done again), staged by TMA and by 16-byte copies, in place too."""
+    sos = designs.butter_lowpass(order, cutoff)
+    n = _five_units_a_strip(dev) + 77 if long else (1 << 20) + 77
+    at = n // 3 + 37
+    x = workloads.normal_f32(6, n)
+    ref = oracle.sosfilt(sos, x)
+    f = _filter(sos)
+    xb = torch.from_numpy(x).to(dev)
+    xb[at] = bad
+    zf = torch.empty(order // 2, 2, device=dev)
+    y = f.run(xb, xb if in_place else None, zf=zf).cpu().numpy()
+    assert f.sync_status() == 0
+    assert oracle.rel_err(y[:at], ref[:at]) < 1e-4
+    assert not np.isfinite(y[at:]).any()
+    assert not np.isfinite(zf.cpu().numpy()).any()
+    f.close()
