@@ -228,3 +228,29 @@ def test_values_that_are_not_finite_in_every_mode(dev, order, cutoff, bad, in_pl
     assert not np.isfinite(y[at:]).any()
     assert not np.isfinite(zf.cpu().numpy()).any()
     f.close()
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("budget", [1, 3000, 30000])
+@pytest.mark.parametrize("order,cutoff", [(2, 0.2), (8, 0.5), (16, 0.05)])
+def test_expired_waits_of_strips_by_tma(dev, order, cutoff, budget, in_place):
+    """A wait that gives up while TMA copies and products are in flight (their own waits have a limit of their
+    own): the run reports SOS_ETIMEOUT, its workspace is as it was, and the next run, on the same block of
+    memory and the same SMs, is right.  With the longer budgets a run may also end in time."""
+    sos = designs.butter_lowpass(order, cutoff)
+    n = _five_units_a_strip(dev) + 77
+    x = torch.randn(n, device=dev, generator=torch.Generator(device=dev).manual_seed(order))
+    good = _filter(sos)
+    want = good.run(x)
+    assert good.sync_status() == 0
+    f = _filter(sos, tuning={"spin_budget_cycles": budget})
+    for _ in range(3):
+        b = x.clone()
+        y = f.run(b, b if in_place else None)
+        status = f.sync_status()
+        assert status == -4 or (budget > 1 and status == 0)
+        if status == 0:
+            assert torch.equal(y, want)
+        assert torch.equal(good.run(x), want) and good.sync_status() == 0
+    f.close()
+    good.close()
