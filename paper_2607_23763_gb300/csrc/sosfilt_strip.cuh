@@ -239,11 +239,6 @@ __device__ __forceinline__ void cp_async_arrive(unsigned long long *bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// `count` arrivals on a shared-memory barrier.
-__device__ __forceinline__ void mbar_arrive_n(unsigned long long *bar, unsigned count) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
 // Barrier of `threads` threads that is also a vote: true when every thread brought true.
 __device__ __forceinline__ bool named_bar_and(int id, int threads, bool ok) {
     unsigned r;
@@ -618,7 +613,7 @@ static_assert(sizeof(StripTail) <= kStripTailBytes, "workspace of a run");
 template <int XS>
 struct StripBars {
     unsigned long long full[XS], xfree[XS], afull[2], afree[2], dfull[kStripDS], dfree[kStripDS], zready[kStripZ], yfull[4], fin;
-    unsigned tmem, strip, last, pad;
+    unsigned tmem, strip, last, stop;
 };
 
 template <int K, bool NORM, int MODE>
@@ -726,48 +721,27 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&zready[0]);
         }
-        if (Sd::TC && P.tma) {
-            // one thread copies, and arrives for all: a unit's phase then waits for nothing but its copies.  The
-            // strip's last unit, where it is not full, comes by 16-byte copies as below
-            unsigned i = 0;
-            for (; w == 0 && i < n_u; ++i) {
-                const unsigned xs = i % XS;
-                if (i >= XS && !strip_wait(&xfree[xs], (i / XS - 1) & 1, budget, p.status)) break;
-                const long long row = r_first + static_cast<long long>(i) * kStripRows;
-                const int rows = r_end - row < kStripRows ? static_cast<int>(r_end - row) : kStripRows;
-                const bool whole = rows == kStripRows && (row + kStripRows) * kStripN <= p.n;
-                if (whole && lane == 0) {
-                    mbar_expect_tx(&full[xs], kStripXBytes);
-                    tma_load_2d(sm + xs * kStripXBytes, &P.tmx, 0, row, &full[xs]);
-                    tma_load_2d(sm + xs * kStripXBytes + kStripHalf, &P.tmx, 32, row, &full[xs]);
-                    mbar_arrive_n(&full[xs], 32 * Sd::LOADERS - 1);
-                }
-                if (!whole) {
-                    const int left = static_cast<int>((p.n < r_end * kStripN ? p.n : r_end * kStripN) - row * kStripN);
-                    const unsigned dst = smem_u32(sm) + xs * kStripXBytes + ((lane & 8) ? kStripHalf : 0);
-#pragma unroll 1
-                    for (int k = 4 * lane, r = lane >> 4; r < kStripRows; k += 2 * kStripN, r += 2) {
-                        const unsigned bytes = left - k >= 4 ? 16u : left > k ? static_cast<unsigned>(4 * (left - k)) : 0u;
-                        cp_async16_s(dst + r * 128 + (((lane ^ r) & 7) << 4), bytes ? p.x + row * kStripN + k : p.x, bytes);
-                    }
-                    cp_async_arrive(&full[xs]);
-                    if (lane == 0) mbar_arrive_n(&full[xs], 32 * (Sd::LOADERS - 1));
-                }
-                trace(i, 16);
-            }
-            // where a wait gave up, the copies in flight land before the block exits, whatever the budget: the
-            // last XS units sit in distinct stages with none issued after them, so theirs are the current phases
-            // (and all are TMA copies: only a strip's last unit can be less than full)
-            if (w == 0 && i < n_u)
-                for (unsigned u = i > XS ? i - XS : 0; u < i; ++u) strip_wait(&full[u % XS], (u / XS) & 1, kStripDrain, p.status);
-        }
-        for (unsigned i = Sd::TC && P.tma ? n_u : 0; i < n_u; ++i) {
+        unsigned i = 0;
+        for (; i < n_u; ++i) {
             const unsigned xs = i % XS;
             if (i >= XS && !strip_wait(&xfree[xs], (i / XS - 1) & 1, budget, p.status)) break;
             const long long base = (r_first + static_cast<long long>(i) * kStripRows) * kStripN;
             const long long avail = (r_end * kStripN < p.n ? r_end * kStripN : p.n) - base;
             const float *x = p.x + base;
             const unsigned dst = smem_u32(sm) + xs * kStripXBytes;
+            if (P.tma && avail >= kStripUnit) {
+                if (w == 0 && lane == 0) {
+                    fence_proxy_async_smem();  // the stage's ordinary reads come before the copy
+                    mbar_expect_tx(&full[xs], kStripXBytes);
+                    const long long row = r_first + static_cast<long long>(i) * kStripRows;
+                    tma_load_2d(sm + xs * kStripXBytes, &P.tmx, 0, row, &full[xs]);
+                    tma_load_2d(sm + xs * kStripXBytes + kStripHalf, &P.tmx, 32, row, &full[xs]);
+                } else {
+                    mbar_arrive(&full[xs]);
+                }
+                if (w == 0) trace(i, 16);
+                continue;
+            }
             if (P.x_aligned) {
                 // 16-byte copies: lane = (row parity, chunk of the row); row 8m + 2k + parity has the chunk at
                 // (chunk ^ parity ^ 2k) & 7
@@ -807,6 +781,19 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             if (w == 0) trace(i, 16);
         }
         cp_async_wait_all();
+        if (Sd::TC && P.tma) {
+            // where a wait gave up, the copies in flight land before the block exits, under a limit of their own: the
+            // warps that issued none stopped anywhere, and arrive for what warp 0 had issued; its last XS units sit
+            // in distinct stages with none issued after them, so theirs are the current phases
+            if (w == 0 && lane == 0) bars.stop = i;
+            named_bar_sync(13, 32 * Sd::LOADERS);
+            const unsigned stop = bars.stop;
+#pragma unroll 1
+            for (; i < stop; ++i) mbar_arrive(&full[i % XS]);
+            if (w == 0 && stop < n_u)
+#pragma unroll 1
+                for (i = stop > XS ? stop - XS : 0; i < stop; ++i) strip_wait(&full[i % XS], (i / XS) & 1, kStripDrain, p.status);
+        }
     } else if (Sd::TC && warp == 1) {
         // ------------------------------------------------------------------ products
         load_tables();
@@ -897,8 +884,6 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 }
                 tc_wait_st();
                 tc_fence_before();
-                // the unit's samples have been read, by ordinary loads, before a TMA copy overwrites the stage
-                if (P.tma && h == 1) fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&afull[h]);
             }
@@ -1147,10 +1132,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                         for (int k = 0; k < KK; ++k) tc_mma_ts(d, d + 64 + 8 * k, tc_sdesc(h + 32 * k), i64, 1u, go);
                         tc_commit_if(&bars.yfull[wg], go);
                     }
-                    if (!strip_wait(&bars.yfull[wg], y_par, budget, p.status)) {
-                        dead = true;
-                        strip_wait(&bars.yfull[wg], y_par, kStripDrain, p.status);  // before tensor memory is released
-                    }
+                    if (!strip_wait(&bars.yfull[wg], y_par, budget, p.status)) dead = true;
                     y_par ^= 1;
                     tc_fence_after();
                 } else {
@@ -1306,6 +1288,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 }
             }
         }
+        // a wait for the last products gave up: they end before tensor memory is released
+        if (Sd::MM && dead) strip_wait(&bars.yfull[wg], y_par ^ 1, kStripDrain, p.status);
     }
     if (Sd::MM && P.tma && warp >= 8 && lane == 0) bulk_wait0();  // the outputs are written
     if (Sd::TC) tc_fence_before();
