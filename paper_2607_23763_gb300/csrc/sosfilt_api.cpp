@@ -659,9 +659,12 @@ sos_status build_tc(sos_filter *f, LanePass &ps, bool nearest) {
 // the zero-input transition over h rows, Q^h, rounds to zero in float32 (is below 2^-150) and so does every
 // later one.  A later power is Q^h Q^j, so the entries of Q^h are held below 2^-150 / (S G), G the largest
 // entry met on the way (a cascade's transition may grow before it decays; 16 times it, for the powers not
-// formed).  Found by binary lifting over the powers Q^(2^k); 0 if 2^14 rows are not enough.
+// formed).  Found by binary lifting over the powers Q^(2^k); 0 if kStripMemoryRows are not enough (a pole
+// radius of 0.9996 and more), which is as far as strip_noise looks.
+constexpr int kStripMemoryRows = 1 << 12;
 int strip_memory(const DMat &M1) {
-    constexpr int kBits = 14;
+    constexpr int kBits = 12;
+    static_assert(kStripMemoryRows == 1 << kBits);
     std::vector<DMat> q{dpow(M1, 64)};
     for (int k = 1; k < kBits; ++k) q.push_back(dmul(q.back(), q.back()));
     double G = 1.0;
@@ -684,10 +687,15 @@ int strip_memory(const DMat &M1) {
     return h + 1 < (1 << kBits) ? h + 1 : 0;
 }
 
+// Cascades above this keep the lookback kernels, whose outputs their users have: where rounding is amplified
+// this much two float32 evaluations differ visibly (order-16 resonators at radius 0.999: noise 3e-5, 3e-5
+// between the kernels' outputs, each 2.3e-5 from float64).
+constexpr double kStripNoise = 1e-5;
+
 // How much a cascade amplifies float32 rounding: the error (2-norm over 2-norm of the output) of its
-// sections run one after the other in float32, in direct-form-I order with fused multiply-adds, on 2048
-// samples of fixed noise.
-double float32_noise(const sos_filter *f) {
+// sections run one after the other in float32, in direct-form-I order with fused multiply-adds, on fixed
+// noise, counted from sample `from` on.  Ends early where the noise is past doubt above kStripNoise.
+double float32_noise(const sos_filter *f, int samples, int from) {
     const int K = f->K;
     std::vector<float> c(4 * static_cast<size_t>(K)), h(2 * static_cast<size_t>(K + 1), 0.f);
     std::vector<double> d(4 * static_cast<size_t>(K)), hd(2 * static_cast<size_t>(K + 1), 0.0);
@@ -702,9 +710,9 @@ double float32_noise(const sos_filter *f) {
             c[4 * k + j] = static_cast<float>(v[j]);
         }
     }
-    double err = 0.0, sum = 0.0;
+    double err = 0.0, sum = 0.0, err_all = 0.0, sum_all = 0.0;
     uint32_t seed = 12345;
-    for (int i = 0; i < 2048; ++i) {
+    for (int i = 0; i < samples; ++i) {
         double u = 0.0;  // four uniforms: variance 1/3
         for (int r = 0; r < 4; ++r) {
             seed = seed * 1664525u + 1013904223u;
@@ -730,16 +738,38 @@ double float32_noise(const sos_filter *f) {
         h[2 * K] = v;
         hd[2 * K + 1] = hd[2 * K];
         hd[2 * K] = w;
-        err += (v - w) * (v - w);
-        sum += w * w;
+        err_all += (v - w) * (v - w);
+        sum_all += w * w;
+        if (i >= from) {
+            err += (v - w) * (v - w);
+            sum += w * w;
+        }
+        if (i % 2048 == 2047 && err_all > 4.0 * kStripNoise * kStripNoise * sum_all) return std::sqrt(err_all / sum_all);
     }
     return sum > 0.0 ? std::sqrt(err / sum) : 1.0;
 }
 
-// Cascades above this keep the lookback kernels, whose outputs their users have: where rounding is amplified
-// this much two float32 evaluations differ visibly (order-16 resonators at radius 0.999: noise 3e-5, 3e-5
-// between the kernels' outputs, each 2.3e-5 from float64), below it by less than 1e-5 of the signal.
-constexpr double kStripNoise = 1e-5;
+// Finds out whether a cascade's runs may go by strips: its passes' memory, and its float32 noise.  Rounding
+// errors pile up for as long as a cascade remembers, so the noise is taken over a quarter of its memory (26 time
+// constants of its slowest pole), of which the second half counts; over 2048 samples, counted whole, where that
+// is more (13 time constants at least).  One resonator at radius 0.999 reads 1.0e-5 over its first 2048 samples
+// and 2.0e-5 later.  A cascade with a longer memory than strip_memory looks for runs by strips only where a signal
+// is one strip, so over that many samples.
+double strip_noise(sos_filter *f) {
+    constexpr int kLeast = 2048;
+    long long rows = 0;
+    for (LanePass &ps : f->lane[1]) {
+        ps.warm_rows = strip_memory(ps.M1);
+        rows = ps.warm_rows && rows >= 0 ? rows + ps.warm_rows : -1;
+    }
+    if (rows < 0) {
+        for (LanePass &ps : f->lane[1]) ps.warm_rows = 0;
+        return float32_noise(f, sosk::kStripUnit, 0);
+    }
+    const int samples = static_cast<int>(16 * (rows < kStripMemoryRows ? rows : kStripMemoryRows));
+    return samples > kLeast ? float32_noise(f, samples, samples / 2) : float32_noise(f, kLeast, 0);
+}
+
 // Below this noise the default solver's strips take their outputs from the recurrences, from it on from the
 // tensor cores, whose products err by 2e-7 to 3e-7 of the signal whatever the cascade: more than recurrences of
 // this little noise (order 12 at 0.4 Nyquist: 1.7e-7 against 3.1e-7), less than noisier ones (order 16 at
@@ -781,7 +811,6 @@ sos_status build_strip(sos_filter *f, LanePass &ps, LanePass &tc, double noise) 
         }
     }
     ps.gresp.assign(buf.begin() + sosk::kStripImgFloats, buf.end());
-    ps.warm_rows = strip_memory(ps.M1);
     tc.products = kp > sosk::kStripStatesK;
     ps.products = tc.products && noise >= kStripProductsNoise;
     if (!ps.products) {
@@ -1904,7 +1933,7 @@ sos_status sos_filter_create(int n_sections, const double *sos, const float *zi,
     for (int i = 0; i < 4 && st == SOS_OK; ++i)
         st = build_lane(f, i == 0 ? 32 : 64, i == 2 ? sosk::kLaneWide : i == 3 ? sosk::kTcGroups : sosk::kLaneW,
                         f->lane[i]);
-    const double noise = float32_noise(f);
+    const double noise = strip_noise(f);
     const bool strips = noise <= kStripNoise;
     for (size_t i = 0; i < f->lane[3].size() && st == SOS_OK; ++i) {
         st = build_tc(f, f->lane[3][i], strips);

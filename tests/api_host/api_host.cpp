@@ -315,6 +315,23 @@ long long host_lane_layout(int K, long long *out) {
         default: return -1;
     }
 }
+// the strip kernel's fields of a launch (LaneParams<K>): warm_rows, products, whether there are tables at all
+#define STRIP_FIELDS(K)                                                            \
+    case K: {                                                                      \
+        const auto *p = reinterpret_cast<const sosk::LaneParams<K> *>(l.params.data()); \
+        out[0] = p->warm_rows;                                                     \
+        out[1] = p->products;                                                      \
+        out[2] = p->gimg != nullptr;                                               \
+        return 0;                                                                  \
+    }
+int host_strip_fields(int i, int *out) {
+    const Launch &l = g_launches.at(static_cast<size_t>(i));
+    switch (l.K) {
+        STRIP_FIELDS(1) STRIP_FIELDS(2) STRIP_FIELDS(3) STRIP_FIELDS(4)
+        STRIP_FIELDS(5) STRIP_FIELDS(6) STRIP_FIELDS(7) STRIP_FIELDS(8)
+        default: return -1;
+    }
+}
 // byte offsets in CasParams<K, N>: n, G, n_tiles, gain, tab, sec, H, A_tail; returns its size
 #define CAS_OFFS(K, N)                                                                                   \
     if (k == K && n == N) {                                                                              \

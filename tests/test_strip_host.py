@@ -1,0 +1,128 @@
+"""The host code that decides whether a cascade's runs may go by strips (sosfilt_api.cpp, on the CPU against the
+stand-ins of tests/api_host/): the rows after which a state is forgotten, and the cascade's float32 noise."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from workloads import designs
+
+from .test_api_host import _create, lib  # noqa: F401  (a fixture)
+
+ROW = 64
+
+
+def _fields(lib, sos, tuning=None):
+    """(warm-up rows, outputs by products, any tables) of each pass of a run."""
+    f = _create(lib, sos, tuning)
+    x = np.zeros(4096, np.float32)
+    lib.host_reset()
+    assert lib.sos_filter_run(f, x.ctypes.data, x.ctypes.data, x.size, None, None, None) == 0
+    out, got = (ctypes.c_int * 3)(), []
+    for i in range(lib.host_launches()):
+        assert lib.host_strip_fields(i, out) == 0
+        got.append(tuple(out))
+    lib.sos_filter_destroy(f)
+    return got
+
+
+def _transition(sos):
+    """One sample of the transposed-direct-form-II cascade under zero input, [2K][2K]."""
+    S = 2 * len(sos)
+    M = np.zeros((S, S))
+    for j in range(S):
+        z, v = np.zeros(S), 0.0
+        z[j] = 1.0
+        for k, (b0, b1, b2, a1, a2) in enumerate(sos):
+            y = b0 * v + z[2 * k]
+            z[2 * k], z[2 * k + 1] = b1 * v - a1 * y + z[2 * k + 1], b2 * v - a2 * y
+            v = y
+        M[:, j] = z
+    return M
+
+
+def _resonator(sections, radius):
+    return designs.resonator_bank(sections, radius=radius)
+
+
+def _dc_blocker(radius):
+    """A zero at frequency zero and a real pole beside it: quiet however long it remembers."""
+    return np.array([[1.0, -1.0, 0.0, -radius, 0.0]])
+
+
+def _smoother(radius):
+    """A one-pole smoother."""
+    return np.array([[1.0 - radius, 0.0, 0.0, -radius, 0.0]])
+
+
+FORGETFUL = [designs.butter_lowpass(2, 0.2), designs.butter_lowpass(16, 0.05), designs.butter_lowpass(8, 0.5),
+             _resonator(1, 0.99), _resonator(4, 0.98), _smoother(0.9), np.array([[0.5, 0.2, 0.1, 0.0, 0.0]])]
+
+
+@pytest.mark.parametrize("i", range(len(FORGETFUL)))
+def test_a_state_is_forgotten_after_the_warm_up_and_not_long_before(lib, i):  # noqa: F811
+    """After warm_rows rows every entry of the transition, and of every later one, is below 2^-150 (zero in
+    float32); at half of them (the rule is careful by a factor in size, not in time) it is not."""
+    sos = FORGETFUL[i]
+    (rows, _, tables), = _fields(lib, sos)
+    assert tables and 1 <= rows < 4096
+    Q = np.linalg.matrix_power(_transition(sos), ROW)
+    P = np.linalg.matrix_power(Q, rows)
+    for _ in range(64):
+        assert np.abs(P).max() < 2.0 ** -150
+        P = P @ Q
+    if rows > 2:
+        assert np.abs(np.linalg.matrix_power(Q, rows // 2)).max() > 2.0 ** -150
+
+
+@pytest.mark.parametrize("sections,radius", [(1, 0.999), (1, 0.9995), (2, 0.9993), (4, 0.999), (8, 0.999)])
+def test_slow_noisy_cascades_keep_the_lookback(lib, sections, radius):  # noqa: F811
+    """Narrow resonators amplify float32 rounding by more than 1e-5 once their errors have piled up, which takes
+    longer than their first 2048 samples: no strip tables."""
+    assert _settled_noise(_resonator(sections, radius)) > 1e-5
+    assert _fields(lib, _resonator(sections, radius))[0][2] == 0
+
+
+@pytest.mark.parametrize("sos", [_resonator(1, 0.9999), _resonator(4, 0.9998), _smoother(0.9999), _dc_blocker(0.99999)])
+def test_cascades_that_remember_too_long_are_never_warmed_up(lib, sos):  # noqa: F811
+    """Beyond 4096 rows of memory no warm-up is given, whatever the noise over a single strip."""
+    assert _fields(lib, sos)[0][0] == 0
+
+
+@pytest.mark.parametrize("radius", [0.99, 0.999, 0.9995])
+def test_slow_quiet_cascades_still_take_strips(lib, radius):  # noqa: F811
+    (rows, _, tables), = _fields(lib, _dc_blocker(radius))
+    assert tables and rows > 0
+
+
+def test_one_slow_pass_keeps_all_passes_from_strips(lib):  # noqa: F811
+    """Nine sections are two passes; a pole that remembers too long, in either, leaves neither a warm-up."""
+    slow = _smoother(0.9999)
+    for sos in (np.vstack([designs.butter_lowpass(16, 0.1), slow]), np.vstack([slow, designs.butter_lowpass(16, 0.1)])):
+        got = _fields(lib, sos)
+        assert len(got) == 2 and all(rows == 0 for rows, _, _ in got)
+
+
+def _settled_noise(sos):
+    """Float32 direct-form-I error over the output in 2-norms, long after the start (numpy, one rounding per
+    operation)."""
+    rng = np.random.default_rng(5)
+    n, skip = 60000, 30000
+    x = rng.standard_normal(n).astype(np.float32)
+    b0 = float(np.prod(sos[:, 0]))
+    v, w = x * np.float32(b0), x.astype(np.float64) * b0
+    for s in sos:
+        q64 = np.array([s[1] / s[0], s[2] / s[0], -s[3], -s[4]])
+        q = q64.astype(np.float32)
+        y, z = np.zeros(n, np.float32), np.zeros(n)
+        x1 = x2 = y1 = y2 = np.float32(0)
+        X1 = X2 = Y1 = Y2 = 0.0
+        for i in range(n):
+            y0 = v[i] + q[0] * x1 + q[1] * x2 + q[2] * y1 + q[3] * y2
+            x2, x1, y2, y1 = x1, v[i], y1, y0
+            y[i] = y0
+            Z = w[i] + q64[0] * X1 + q64[1] * X2 + q64[2] * Y1 + q64[3] * Y2
+            X2, X1, Y2, Y1 = X1, w[i], Y1, Z
+            z[i] = Z
+        v, w = y, z
+    return float(np.linalg.norm(v[skip:] - w[skip:]) / np.linalg.norm(w[skip:]))
