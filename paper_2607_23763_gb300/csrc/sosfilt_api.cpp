@@ -1097,6 +1097,14 @@ sos_status run_dtcr(sos_filter *f, const float *x, float *y, int64_t n, const fl
     return SOS_OK;
 }
 
+// How a pass cuts its signal into strips (none: it runs the lookback kernel; tc: that is the tensor-core one).
+sosk::StripCut strips_of(const sos_filter *f, const LanePass &ps, const float *x, long long n, bool tc) {
+    sosk::StripCut c{};
+    const bool odd = reinterpret_cast<uintptr_t>(x) % 16 != 0;
+    if (!ps.gimg || !sosk::strip_cut(ps.kp, ps.products, odd, tc, n, ps.warm_rows, sm_count(f->device), c)) c = {};
+    return c;
+}
+
 // ---- skewed-pass PH kernel (sosfilt_lane.cuh)
 template <int K, int N, int W, bool TC = false>
 sos_status launch_lane_pass(sos_filter *f, LanePass &ps, const float *x, float *y, long long n, long long G,
@@ -1148,7 +1156,7 @@ sos_status launch_lane_pass(sos_filter *f, LanePass &ps, const float *x, float *
         p->gimg = ps.gimg;
         p->gtail = ps.gtail;
         p->gresp = ps.gresp.data();
-        p->warm_rows = ps.warm_rows;
+        p->cut = strips_of(f, ps, x, n, TC);
         p->norm = f->norm ? 1 : 0;
         p->tail = sc ? sc->tail : reinterpret_cast<unsigned *>(f->d_ticket + 2);
     }

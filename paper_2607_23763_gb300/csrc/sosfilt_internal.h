@@ -3,6 +3,8 @@
 #pragma once
 #include <cstdint>
 
+#include "sosfilt_strip_rule.h"
+
 #include <cuda_runtime.h>
 
 namespace sosk {
@@ -137,8 +139,7 @@ constexpr int kLaneWide = 10;  // the wide variant at N = 64: 10 groups per tile
 
 // ---- PH kernel over strips (sosfilt_strip.cuh): one strip of consecutive samples per block, for cascades
 // whose memory is finite in float32
-constexpr int kStripUnit = 8192;        // samples of a unit of its work: 128 rows of 64
-constexpr int kStripMax = 256;          // strips of a run (at most one per SM)
+constexpr int kStripUnit = kStripN * kStripRows;  // samples of a unit of its work
 constexpr size_t kStripTailBytes = 128 + 4 * kStripMax;  // a run's workspace, zero between runs
 constexpr int kStripImgFloats = 2048;   // tensor-core image of the state responses (8 KB)
 // up to this many sections the outputs come from the recurrences (2^28 samples at order 2: 330 to 360 us,
@@ -176,12 +177,12 @@ struct LaneParams {
     // blocks (k, j), j < k, of the lane transition M_N, row-major 2x2 at k (k - 1) / 2 + j
     float4 MX[K > 1 ? K * (K - 1) / 2 : 1];
     float A_tail[2 * K * (K + 1)];  // packed cascade transition over m_last + 1 samples
-    // the strip kernel's (kernels at N = 64): the tensor cores' operand image (kStripImgFloats or, with
-    // outputs, kTcImageBytes) and the state responses in float32 ([2K][64]), rows of 64 samples until the cascade's state is forgotten in float32 (0: not
-    // within 2^14), whether the tensor cores form the outputs, b0-normalized, workspace (nullptr: none)
+    // the strip kernel's (kernels at N = 64): how the signal is cut (no strips: the pass runs the lookback kernel),
+    // the tensor cores' operand image (kStripImgFloats or, with outputs, kTcImageBytes) and the state responses in
+    // float32 ([2K][64]), whether the tensor cores form the outputs, b0-normalized, workspace
+    StripCut cut;
     const float *gimg, *gtail;
     const float *gresp;  // gtail in host memory
-    int warm_rows;
     int products;
     int norm;
     unsigned *tail;
@@ -305,7 +306,7 @@ struct BatchAllParams {
 cudaError_t launch_batch_all(const BatchAllParams &p, long long grid, cudaStream_t s);
 int batch_all_blocks_per_sm();
 
-// Runs a pass by strips where that is the better way (returns true, with the launch's status in err);
+// Runs a pass by strips if its signal is cut into any (returns true, with the launch's status in err);
 // otherwise false, and nothing was launched.  grid: what the caller's own kernel would use, added with
 // the tile count to the eager launches' ticket counter as that kernel would leave it.
 template <int K>

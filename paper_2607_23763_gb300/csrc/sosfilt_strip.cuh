@@ -34,7 +34,6 @@
 // Without the tensor cores warps 0-7 all load.
 // Every wait is bounded by the spin budget.
 #pragma once
-#include <atomic>
 #include <cstring>
 
 #include "sosfilt_lane.cuh"
@@ -42,9 +41,6 @@
 
 namespace sosk {
 
-constexpr int kStripN = 64;                        // samples per row
-constexpr int kStripRows = 128;                    // rows per unit (four groups of 32 lanes)
-static_assert(kStripUnit == kStripN * kStripRows, "unit geometry");
 constexpr int kStripXBytes = kStripUnit * 4;       // one staged unit: two column halves of 16 KB
 constexpr int kStripHalf = kStripXBytes / 2;
 constexpr int kStripDS = 4;                        // accumulator slots, ahead of the operand buffers
@@ -114,54 +110,6 @@ struct StripDims {
     static constexpr size_t SMEM = OFF_BAR + kStripBars;
 };
 
-// How a signal is cut into strips.
-struct StripCut {
-    long long n_rows;
-    int strip_rows;    // rows per strip (the last strip may be shorter)
-    int n_strips;      // strips = thread blocks
-    int warm_rows;     // rows a strip starts early
-};
-
-// A signal of n samples in strips, at most one per SM.  A signal of one unit is one strip; a strip is at
-// least half a unit, and no shorter than its warm-up, so that a warm-up reaches into one neighbour only.
-// False where strips are not taken: the cascade remembers for longer than a strip is (its warm-up would
-// then cost as much as the strip; two units of it are taken even so, since they cost less than a chain of
-// lookbacks).
-inline bool strip_cut(long long n, int warm_rows, StripCut &c) {
-    static std::atomic<int> known[64];  // SMs of a device, 0: not asked yet
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-    int sms = known[dev].load(std::memory_order_relaxed);
-    if (!sms) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
-        known[dev].store(sms, std::memory_order_relaxed);
-    }
-    if (sms > kStripMax) sms = kStripMax;
-    c.n_rows = (n + kStripN - 1) / kStripN;
-    c.warm_rows = warm_rows;
-    long long per = (c.n_rows + sms - 1) / sms;
-    if (per > (1LL << 30)) return false;
-    const long long most = per > 2 * kStripRows ? per : 2 * kStripRows;
-    if (c.n_rows <= kStripRows) {
-        per = c.n_rows;
-        c.warm_rows = 0;
-    } else {
-        if (warm_rows < 1 || warm_rows > most) return false;
-        if (per < kStripRows / 2) per = kStripRows / 2;
-        if (per < warm_rows) per = warm_rows;
-    }
-    c.strip_rows = static_cast<int>(per);
-    c.n_strips = static_cast<int>((c.n_rows + per - 1) / per);
-    return true;
-}
-
-// One or two sections: strips of at most this many rows with their warm-up take the terminal states by FMAs
-// (no operands, products or tensor memory on the way: a 4096-sample call is 0.6 of the time in the kernel),
-// longer ones on the tensor cores (2^28 samples at order 2: 329 us against 354).
-constexpr int kStripFmaRows = 4 * kStripRows;
-
-// Rows of the shortest signals of three and more sections taken by strips, and of three or four unaligned.
-constexpr long long kStripLeastRows = 2048, kStripLeastRows4 = 45000;
 // Strips of at least this many rows take TMA copies.
 constexpr int kStripTmaRows = 4 * kStripRows;
 // A signal's full rows of 64 samples as a tensor map, copied in boxes of 32 x box_rows (sosfilt_tc.cu).
@@ -179,7 +127,6 @@ struct StripPairs {
 template <int K, int MODE>
 struct StripParams {
     LaneParams<K> p;
-    StripCut cut;
     int in_place;      // y == x: a strip's tail is stored once the next strip has read it
     int x_aligned, y_aligned;  // 16-byte aligned
     int tma;           // tmx and tmy are set: full units are loaded, full groups' outputs stored by TMA
@@ -640,7 +587,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
     if (tid == 0) {
         // in place, a strip's last rows are stored once the next strip has read them: strips are taken from
         // the last one down, so that the block waited on is running or done
-        bars.strip = P.in_place && P.cut.n_strips > 1 ? P.cut.n_strips - 1 - atomicAdd(&tail->ticket, 1u) : blockIdx.x;
+        bars.strip = P.in_place && p.cut.n_strips > 1 ? p.cut.n_strips - 1 - atomicAdd(&tail->ticket, 1u) : blockIdx.x;
         for (int i = 0; i < XS; ++i) {
             mbar_init(&full[i], 32 * Sd::LOADERS);
             mbar_init(&xfree[i], 4);
@@ -663,14 +610,14 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
     if (Sd::TC) tc_fence_after();
     const unsigned tmem = Sd::TC ? bars.tmem : 0;
     const int strip = static_cast<int>(bars.strip);
-    const long long r_own = static_cast<long long>(strip) * P.cut.strip_rows;
-    const long long r_end = r_own + P.cut.strip_rows < P.cut.n_rows ? r_own + P.cut.strip_rows : P.cut.n_rows;
-    const int n_warm = r_own < P.cut.warm_rows ? static_cast<int>(r_own) : P.cut.warm_rows;
+    const long long r_own = static_cast<long long>(strip) * p.cut.strip_rows;
+    const long long r_end = r_own + p.cut.strip_rows < p.cut.n_rows ? r_own + p.cut.strip_rows : p.cut.n_rows;
+    const int n_warm = r_own < p.cut.warm_rows ? static_cast<int>(r_own) : p.cut.warm_rows;
     // units of 128 rows from r_first on; rows r_first .. r_own - 1 only warm up, rows past r_end are zeros
     const long long r_first = r_own - n_warm;
     const unsigned n_u = static_cast<unsigned>((r_end - r_first + kStripRows - 1) / kStripRows);
     // phase trace (diagnostics; nothing is written without a trace buffer): one item per unit, strip by strip
-    const long long item0 = strip * ((static_cast<long long>(P.cut.strip_rows) + P.cut.warm_rows + kStripRows - 1) / kStripRows);
+    const long long item0 = strip * ((static_cast<long long>(p.cut.strip_rows) + p.cut.warm_rows + kStripRows - 1) / kStripRows);
     auto trace = [&](unsigned i, int slot) {
         if (p.trace && lane == 0 && item0 + i < p.trace_tiles)
             p.trace[static_cast<size_t>(item0 + i) * kTraceSlots + slot] = global_ns();
@@ -995,8 +942,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     if (lane < S) z_buf[((i + 1) % kStripZ) * S + lane] = zn;
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&zready[(i + 1) % kStripZ]);
-                } else if (__any_sync(0xffffffffu, !(fabsf(zn) <= 3.402823466e38f)) && lane == 0 && strip + 1 < P.cut.n_strips) {
-                    atomicMax(&tail->poison, static_cast<unsigned>(P.cut.n_strips - strip));
+                } else if (__any_sync(0xffffffffu, !(fabsf(zn) <= 3.402823466e38f)) && lane == 0 && strip + 1 < p.cut.n_strips) {
+                    atomicMax(&tail->poison, static_cast<unsigned>(p.cut.n_strips - strip));
                 }
             }
             // the unit's first and last own rows; with outputs its four warps stay together for the products
@@ -1037,10 +984,10 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                 unsigned char *X = sm + xs * kStripXBytes;
                 const long long base = R * kStripN;
                 if (q == 0) trace(i, 10);
-                if (p.zf && r_end == P.cut.n_rows && R + 32 >= r_end) {
+                if (p.zf && r_end == p.cut.n_rows && R + 32 >= r_end) {
                     // final state: the last row's samples under zero state, taken across the lanes, plus
                     // the transition of the row's incoming state over them
-                    const int lane_last = static_cast<int>(P.cut.n_rows - 1 - R);
+                    const int lane_last = static_cast<int>(p.cut.n_rows - 1 - R);
                     const int ml = p.m_last;
                     [[maybe_unused]] const int rl = 32 * q + lane_last;
                     float acc[S], zt[S];
@@ -1070,7 +1017,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     if (lane == lane_last) {
                         // with several strips the block that finishes last hands the state over, since zf
                         // may be the array another strip reads its initial state from
-                        float *zf = P.cut.n_strips > 1 ? tail->zf : p.zf;
+                        float *zf = p.cut.n_strips > 1 ? tail->zf : p.zf;
 #pragma unroll
                         for (int s = 0; s < S; ++s) zf[s] = (acc[s] + zt[s]) * p.sec[s >> 1].zscale_inv;
                     }
@@ -1150,7 +1097,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     __syncwarp();
                 }
                 if (q == 0) trace(i, 11);
-                if (P.in_place && own && strip + 1 < P.cut.n_strips && R + 32 > r_end - P.cut.warm_rows) {
+                if (P.in_place && own && strip + 1 < p.cut.n_strips && R + 32 > r_end - p.cut.warm_rows) {
                     const long long t0 = clock64();
                     bool seen = false, late = false;
                     while (!seen && !late) {
@@ -1303,7 +1250,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
     // is not finite (the following strips, which did not see it, become NaN as the recurrence would
     // leave them); the workspace is left as it was found
     if (blockIdx.x == 0 && tid == 0 && P.host_tickets) atomicAdd(p.ticket, P.host_tickets);
-    if (P.cut.n_strips == 1) return;
+    if (p.cut.n_strips == 1) return;
     if (tid == 0) {
         __threadfence();
         bars.last = atomicAdd(&tail->done, 1u) + 1 == gridDim.x;
@@ -1314,11 +1261,11 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
     const unsigned poison = *reinterpret_cast<volatile unsigned *>(&tail->poison);
     const float nan = __uint_as_float(0x7fffffffu);
     if (poison) {
-        const long long from = static_cast<long long>(P.cut.n_strips - poison + 1) * P.cut.strip_rows * kStripN;
+        const long long from = static_cast<long long>(p.cut.n_strips - poison + 1) * p.cut.strip_rows * kStripN;
         for (long long k = from + tid; k < p.n; k += Sd::THREADS) p.y[k] = nan;
     }
     if (p.zf && tid < S) p.zf[tid] = poison ? nan : *reinterpret_cast<volatile float *>(&tail->zf[tid]);
-    for (int k = tid; k < P.cut.n_strips; k += Sd::THREADS) tail->flag[k] = 0;
+    for (int k = tid; k < p.cut.n_strips; k += Sd::THREADS) tail->flag[k] = 0;
     __syncthreads();
     if (tid == 0) tail->ticket = tail->poison = tail->done = 0;
 }
@@ -1333,25 +1280,24 @@ cudaError_t launch_strip_one(const StripParams<K, MODE> &P, cudaStream_t s) {
     auto kern = sos_strip_kernel<K, NORM, MODE>;
     cudaError_t e = raise_smem_once(g_strip_once<K, NORM, MODE>, kern, Sd::SMEM);
     if (e != cudaSuccess) return e;
-    kern<<<static_cast<unsigned>(P.cut.n_strips), Sd::THREADS, Sd::SMEM, s>>>(P);
+    kern<<<static_cast<unsigned>(P.p.cut.n_strips), Sd::THREADS, Sd::SMEM, s>>>(P);
     return cudaGetLastError();
 }
 
 template <int K, int MODE>
-cudaError_t launch_strip_mode(const LaneParams<K> &p, const StripCut &cut, long long grid, cudaStream_t s) {
+cudaError_t launch_strip_mode(const LaneParams<K> &p, long long grid, cudaStream_t s) {
     StripParams<K, MODE> P;
     std::memset(static_cast<void *>(&P), 0, sizeof(P));
     P.p = p;
     if constexpr (MODE == kStripOutputs)
         for (auto &b : P.p.MX) b = make_float4(b.x, b.z, b.y, b.w);  // by columns (scan2)
-    P.cut = cut;
     P.in_place = p.x == p.y;
     P.x_aligned = reinterpret_cast<uintptr_t>(p.x) % 16 == 0;
     P.y_aligned = reinterpret_cast<uintptr_t>(p.y) % 16 == 0;
     P.host_tickets = static_cast<unsigned long long>(p.n_tiles + grid);
     if constexpr (MODE != kStripFma) {
         // the tensor maps cost a call about a microsecond on the host: for strips of several units
-        if (P.x_aligned && P.y_aligned && cut.strip_rows >= kStripTmaRows)
+        if (P.x_aligned && P.y_aligned && p.cut.strip_rows >= kStripTmaRows)
             P.tma = strip_rows_map(&P.tmx, p.x, p.n / kStripN, kStripRows) &&
                     strip_rows_map(&P.tmy, p.y, p.n / kStripN, 32);
     }
@@ -1374,32 +1320,19 @@ cudaError_t launch_strip_mode(const LaneParams<K> &p, const StripCut &cut, long 
 
 template <int K>
 bool launch_strip_k(const LaneParams<K> &p, long long grid, cudaStream_t s, cudaError_t &err) {
-    StripCut cut;
-    if (!p.tail || !p.gimg || !strip_cut(p.n, p.warm_rows, cut)) return false;
-    if constexpr (K > kStripStatesK) {
-        // short signals: the strip kernel's start (operands, products) costs more than a few tiles' lookback
-        // (order 6, 65536 samples: 12.4 us against 10.5; 200000: 12.5 against 12.5; order 16: 14.5 against 16.5
-        // and 15 against 20), the more so where the samples come 4 bytes at a time (order 8, 2.2 M samples: 20.7
-        // against 18.6; 3 M: 20.7 against 22.3)
-        const bool aligned = reinterpret_cast<uintptr_t>(p.x) % 16 == 0;
-        if (cut.n_rows < (aligned || K > 4 ? kStripLeastRows : kStripLeastRows4)) return false;
-    }
+    if (!p.cut.n_strips) return false;
     if constexpr (K <= kStripStatesK) {
-        if (cut.strip_rows + cut.warm_rows <= kStripFmaRows) {
-            err = launch_strip_mode<K, kStripFma>(p, cut, grid, s);
+        if (p.cut.fma) {
+            err = launch_strip_mode<K, kStripFma>(p, grid, s);
             return true;
         }
+    } else if (p.products) {
+        err = launch_strip_mode<K, kStripOutputs>(p, grid, s);
+        return true;
     }
-    if constexpr (K > kStripStatesK) {
-        if (p.products) {
-            err = launch_strip_mode<K, kStripOutputs>(p, cut, grid, s);
-            return true;
-        }
-    }
-    err = launch_strip_mode<K, kStripStates>(p, cut, grid, s);
+    err = launch_strip_mode<K, kStripStates>(p, grid, s);
     return true;
 }
-
 
 #define SOSK_STRIP_INST(k)                                                                           \
     template <>                                                                                      \

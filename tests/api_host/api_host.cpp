@@ -315,14 +315,14 @@ long long host_lane_layout(int K, long long *out) {
         default: return -1;
     }
 }
-// the strip kernel's fields of a launch (LaneParams<K>): warm_rows, products, whether there are tables at all
-#define STRIP_FIELDS(K)                                                            \
-    case K: {                                                                      \
+// the strip kernel's fields of a launch (LaneParams<K>): strips, rows a strip, warm-up rows, by FMAs, products,
+// whether there are tables at all
+#define STRIP_FIELDS(K)                                                                 \
+    case K: {                                                                           \
         const auto *p = reinterpret_cast<const sosk::LaneParams<K> *>(l.params.data()); \
-        out[0] = p->warm_rows;                                                     \
-        out[1] = p->products;                                                      \
-        out[2] = p->gimg != nullptr;                                               \
-        return 0;                                                                  \
+        const int v[] = {p->cut.n_strips, p->cut.strip_rows, p->cut.warm_rows, p->cut.fma, p->products, p->gimg != nullptr}; \
+        std::memcpy(out, v, sizeof v);                                                  \
+        return 0;                                                                       \
     }
 int host_strip_fields(int i, int *out) {
     const Launch &l = g_launches.at(static_cast<size_t>(i));
@@ -331,6 +331,14 @@ int host_strip_fields(int i, int *out) {
         STRIP_FIELDS(5) STRIP_FIELDS(6) STRIP_FIELDS(7) STRIP_FIELDS(8)
         default: return -1;
     }
+}
+// strip_cut of a pass: 1 and {strips, rows a strip, warm-up rows, by FMAs}, or 0
+int host_strip_cut(int K, int products, int odd, int tc, long long n, int warm_rows, int sms, int *out) {
+    sosk::StripCut c{};
+    if (!sosk::strip_cut(K, products != 0, odd != 0, tc != 0, n, warm_rows, sms, c)) return 0;
+    const int v[] = {c.n_strips, c.strip_rows, c.warm_rows, c.fma};
+    std::memcpy(out, v, sizeof v);
+    return 1;
 }
 // byte offsets in CasParams<K, N>: n, G, n_tiles, gain, tab, sec, H, A_tail; returns its size
 #define CAS_OFFS(K, N)                                                                                   \

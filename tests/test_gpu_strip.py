@@ -173,9 +173,11 @@ def test_streams_and_filters_at_once(dev):
         f.close()
 
 
-def _five_units_a_strip(dev):
-    """Samples of a signal whose strips are long enough (512 rows and more) for TMA copies."""
-    return 5 * torch.cuda.get_device_properties(dev).multi_processor_count * UNIT
+def _long(dev, order):
+    """Samples of a signal whose strips take TMA copies: 512 rows and more, and at one and two sections more than
+    what is done without the tensor cores."""
+    rows = {2: 3400, 4: 12300}.get(order, 640)
+    return rows * torch.cuda.get_device_properties(dev).multi_processor_count * ROW
 
 
 # what forms the outputs: recurrences of one and two sections, in pairs, one at a time; products (both solvers)
@@ -188,7 +190,7 @@ def test_strips_by_tma(dev, order, cutoff, solver, tail):
     """Strips long enough for TMA copies, with an initial and a final state: against the oracle, and the run in
     place, with the final state over the initial one, bit for bit the same."""
     sos = designs.butter_lowpass(order, cutoff)
-    n = _five_units_a_strip(dev) + tail
+    n = _long(dev, order) + tail
     x = workloads.normal_f32(11 + order, n)
     zi = (0.01 * np.random.default_rng(order).standard_normal((order // 2, 2))).astype(np.float32)
     ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
@@ -214,7 +216,7 @@ def test_values_that_are_not_finite_in_every_mode(dev, order, cutoff, bad, in_pl
     """The same for each way of forming the outputs (order 16 at 0.05: products, whose rows with such samples are
     done again), staged by TMA and by 16-byte copies, in place too."""
     sos = designs.butter_lowpass(order, cutoff)
-    n = _five_units_a_strip(dev) + 77 if long else (1 << 20) + 77
+    n = _long(dev, order) + 77 if long else (1 << 20) + 77
     at = n // 3 + 37
     x = workloads.normal_f32(6, n)
     ref = oracle.sosfilt(sos, x)
@@ -238,7 +240,7 @@ def test_expired_waits_of_strips_by_tma(dev, order, cutoff, budget, in_place):
     own): the run reports SOS_ETIMEOUT, its workspace is as it was, and the next run, on the same block of
     memory and the same SMs, is right.  With the longer budgets a run may also end in time."""
     sos = designs.butter_lowpass(order, cutoff)
-    n = _five_units_a_strip(dev) + 77
+    n = _long(dev, order) + 77
     x = torch.randn(n, device=dev, generator=torch.Generator(device=dev).manual_seed(order))
     good = _filter(sos)
     want = good.run(x)
@@ -254,3 +256,50 @@ def test_expired_waits_of_strips_by_tma(dev, order, cutoff, budget, in_place):
         assert torch.equal(good.run(x), want) and good.sync_status() == 0
     f.close()
     good.close()
+
+
+@pytest.mark.parametrize("ox,oy", [(1, 1), (0, 0), (3, 0), (0, 2)])
+@pytest.mark.parametrize("rows", [300, 1300])
+@pytest.mark.parametrize("order", [2, 4])
+def test_strips_of_many_units_by_fmas(dev, order, rows, ox, oy):
+    """One and two sections without the tensor cores, strips of several units: misaligned signals of any length and
+    aligned ones of up to a few thousand rows a strip, with states, in place too."""
+    sos = designs.butter_lowpass(order, 0.05)
+    n = rows * torch.cuda.get_device_properties(dev).multi_processor_count * ROW + 77
+    x = workloads.normal_f32(21 + order, n)
+    zi = (0.01 * np.random.default_rng(order).standard_normal((order // 2, 2))).astype(np.float32)
+    ref, zref = oracle.sosfilt(sos, x, zi=zi.astype(np.float64), return_state=True)
+    f = _filter(sos)
+    xd = torch.empty(n + ox, device=dev)[ox:]
+    xd.copy_(torch.from_numpy(x))
+    y = torch.full((n + oy + 8,), 7.0, device=dev)
+    z, zf = torch.from_numpy(zi).to(dev), torch.empty(order // 2, 2, device=dev)
+    f.run(xd, y[oy:oy + n], zi=z, zf=zf)
+    assert f.sync_status() == 0
+    assert bool((y[:oy] == 7.0).all()) and bool((y[oy + n:] == 7.0).all())
+    assert oracle.rel_err(y[oy:oy + n].cpu().numpy(), ref) < 1e-4
+    assert np.abs(zf.cpu().numpy() - zref).max() < 1e-4 * np.abs(zref).max()
+    f.run(xd, xd, zi=z, zf=z)
+    assert f.sync_status() == 0
+    assert torch.equal(xd, y[oy:oy + n]) and torch.equal(z, zf)
+    f.close()
+
+
+@pytest.mark.parametrize("order,cutoff", [(2, 0.2), (4, 0.1), (6, 0.5), (6, 0.1), (8, 0.1), (10, 0.1), (12, 0.05), (16, 0.05)])
+@pytest.mark.parametrize("n", [1 << 17, (1 << 18) + 5, 1 << 20, 3 << 20, 6 << 20])
+def test_both_ways_agree_where_the_rule_changes(dev, order, cutoff, n):
+    """Lengths around the lines between strips and lookback, aligned, misaligned and with the tensor-core solver: each
+    against the lookback kernel of ten groups a tile, which never takes strips."""
+    sos = designs.butter_lowpass(order, cutoff)
+    x = torch.randn(n + 4, device=dev, generator=torch.Generator(device=dev).manual_seed(n + order))
+    b = _filter(sos, tuning={"solver": 2, "groups_per_cta": 10})
+    for solver in (0, 4):
+        a = _filter(sos, tuning={"solver": solver})
+        for o in (0, 1, 2):
+            za, zb = torch.empty(order // 2, 2, device=dev), torch.empty(order // 2, 2, device=dev)
+            ya, yb = a.run(x[o:o + n], zf=za), b.run(x[o:o + n], zf=zb)
+            assert a.sync_status() == 0 and b.sync_status() == 0
+            assert float((ya - yb).abs().max()) < 2e-5 * float(yb.abs().max())
+            assert float((za - zb).abs().max()) < 2e-5 * float(zb.abs().max())
+        a.close()
+    b.close()
