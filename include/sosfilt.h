@@ -442,18 +442,20 @@ sos_status sos_server_replay(sos_server *s, int64_t n_req, const int32_t *stream
  * (4 groups of two warps per tile) and PH factorization on the tensor cores (8
  * groups per tile); L = 32 threads per group (thread group)
  * throughout -- for 1 to 8 sections and lengths 2^16, 2^20, 2^24 and 2^28 (up to
- * 2^max_log2n, 0 = 28), and keep the fastest per (section count, length).
+ * 2^max_log2n, 0 = 28), and keep the fastest per (section count, length): once for
+ * runs that a PH solver takes by strips, once for those that keep the lookback kernels
+ * (a cascade that remembers too long or amplifies rounding too much, a short signal).
  * Afterwards every run of a filter created with default tuning (all fields 0)
- * uses the choice for its section count and the nearest length.  Synchronous;
+ * uses the choice for its kind, its section count and the nearest length.  Synchronous;
  * allocates and frees 2^(max_log2n + 3) bytes of device memory; a second or two.
  *   report  NULL, or host float[8][4][6] receiving the measured GS/s
  *           (sections, length 2^16..2^28, candidate CR32/CR64/PH/DTCR/PH with
- *           10 groups per tile/PH on the tensor cores)
+ *           10 groups per tile/PH on the tensor cores) of a cascade that takes strips
  */
 sos_status sos_autotune(int max_log2n, float *report);
 
-/* The autotuned choice for K sections and n samples on the current device:
- * solver (SOS_SOLVER_CR / SOS_SOLVER_PH / SOS_SOLVER_DTCR / SOS_SOLVER_TC) and N; both
+/* The autotuned choice for K sections and n samples on the current device, for a run
+ * that a PH solver takes by strips: solver (SOS_SOLVER_CR / SOS_SOLVER_PH / SOS_SOLVER_DTCR / SOS_SOLVER_TC) and N; both
  * 0 if no autotuning ran. */
 sos_status sos_autotune_choice(int n_sections, int64_t n, int *solver, int *N);
 /* The same with the groups per tile of a PH choice (7 or 10; 8 for SOS_SOLVER_TC; 0 for the

@@ -1276,10 +1276,13 @@ int solver_of(const sos_filter *f) {
 constexpr int kTuneBuckets = 4;                       // n around 2^16, 2^20, 2^24, 2^28
 constexpr int kTuneLog2[kTuneBuckets] = {16, 20, 24, 28};
 constexpr int kTuneCand = 6;  // candidates: CR N = 32, CR N = 64, PH (7 groups), DTCR, PH (10 groups), TC
+// Each for runs that either PH solver takes by strips ([0]) and for runs that both leave to the lookback kernels
+// ([1]: cascades that remember for too long or amplify rounding too much, and short signals): the two solvers' times
+// differ between the kinds (order 16, 2^28 samples: by strips 428 us both, lookback 1180 and 927).
 struct TuneTable {
     bool valid = false;
-    unsigned char best[8][kTuneBuckets] = {};         // candidate index
-    float gss[8][kTuneBuckets][kTuneCand] = {};       // measured GS/s
+    unsigned char best[2][8][kTuneBuckets] = {};      // candidate index
+    float gss[2][8][kTuneBuckets][kTuneCand] = {};    // measured GS/s
 };
 std::mutex g_tune_mu;
 TuneTable g_tune[64];
@@ -1335,13 +1338,20 @@ int tune_bucket(int64_t n) {
     return b;
 }
 
-bool tuned_choice(int device, int K, int64_t n, int *solver, int *N, int *W) {
+bool tuned_choice(int device, int K, int64_t n, bool strips, int *solver, int *N, int *W) {
     if (device < 0 || device >= 64) return false;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_tune[device].valid) return false;
     const int k = (K > sosk::kMaxPass ? sosk::kMaxPass : K) - 1;
-    candidate(g_tune[device].best[k][tune_bucket(n)], solver, N, W);
+    candidate(g_tune[device].best[strips ? 0 : 1][k][tune_bucket(n)], solver, N, W);
     return true;
+}
+
+// Whether a run goes by strips under one of the PH solvers (its first pass, which is the longest cascade).
+bool runs_by_strips(const sos_filter *f, const float *x, const float *y, int64_t n) {
+    const bool aligned = (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) % 16 == 0;
+    return strips_of(f, f->lane[1].front(), x, n, false).n_strips ||
+           (aligned && strips_of(f, f->lane[3].front(), x, n, true).n_strips);
 }
 
 sos_status run_impl(sos_filter *f, const float *x, float *y, int64_t n, const float *zi, float *zf, cudaStream_t s) {
@@ -1361,7 +1371,7 @@ sos_status run_impl(sos_filter *f, const float *x, float *y, int64_t n, const fl
     if (!t.N && !t.carry && !t.solver && !t.lookback_width && !t.groups_per_cta) {
         // all defaults: the autotuned choice for this section count and length, if there is one
         int solver = 0, N = 0, W = 0;
-        if (tuned_choice(f->device, f->K, n, &solver, &N, &W)) {
+        if (tuned_choice(f->device, f->K, n, runs_by_strips(f, x, y, n), &solver, &N, &W)) {
             if (solver == SOS_SOLVER_PH) return run_lane(f, x, y, n, zi, zf, s, N, W);
             if (solver == SOS_SOLVER_DTCR) return run_dtcr(f, x, y, n, zi, zf, s);
             if (solver == SOS_SOLVER_TC) return run_tc(f, x, y, n, zi, zf, s);
@@ -2217,18 +2227,25 @@ sos_status sos_autotune(int max_log2n, float *report) {
     }
     TuneTable tt;
     sos_status rc = SOS_OK;
-    for (int K = 1; K <= sosk::kMaxPass && rc == SOS_OK; ++K) {
-        // a stable cascade of K sections (the timing does not depend on the coefficients' values)
+    // per section count a cascade that forgets its state within some ten rows, then one that never does in time, for
+    // which only the candidates that take strips are timed again
+    for (int i = 0; i < 2 * sosk::kMaxPass && rc == SOS_OK; ++i) {
+        const int K = i % sosk::kMaxPass + 1, kind = i / sosk::kMaxPass;
         std::vector<double> sos(5 * K);
         for (int k = 0; k < K; ++k) {
-            const double r = 0.9 + 0.01 * k, th = 0.2 + 0.05 * k;
+            const double r = kind ? 0.9999 : 0.9 + 0.01 * k, th = 0.2 + 0.05 * k;
             const double c[5] = {0.05, 0.1, 0.05, -2.0 * r * std::cos(th), r * r};
             std::memcpy(&sos[5 * k], c, sizeof c);
         }
+        auto &gss = tt.gss[kind][K - 1];
         for (int c = 0; c < kTuneCand && rc == SOS_OK; ++c) {
             sos_tuning t{};
             int solver = 0, N = 0, W = 0;
             candidate(c, &solver, &N, &W);
+            if (kind && !(solver == SOS_SOLVER_TC || (solver == SOS_SOLVER_PH && W == sosk::kLaneW))) {
+                for (int b = 0; b < kTuneBuckets; ++b) gss[b][c] = tt.gss[0][K - 1][b][c];
+                continue;
+            }
             t.solver = solver;
             t.N = N;
             t.groups_per_cta = solver == SOS_SOLVER_TC ? 0 : W;  // the tensor-core tile is fixed
@@ -2238,7 +2255,7 @@ sos_status sos_autotune(int max_log2n, float *report) {
             if (rc != SOS_OK) break;
             for (int b = 0; b < kTuneBuckets && rc == SOS_OK; ++b) {
                 if (kTuneLog2[b] > top) {
-                    tt.gss[K - 1][b][c] = tt.gss[K - 1][b > 0 ? b - 1 : 0][c];
+                    gss[b][c] = gss[b > 0 ? b - 1 : 0][c];
                     continue;
                 }
                 const int64_t n = 1LL << kTuneLog2[b];
@@ -2254,15 +2271,15 @@ sos_status sos_autotune(int max_log2n, float *report) {
                 if (rc == SOS_OK && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) !=
                                                                                      cudaSuccess))
                     rc = SOS_ECUDA;
-                if (rc == SOS_OK) tt.gss[K - 1][b][c] = ms > 0.f ? static_cast<float>(n) * reps / ms / 1e6f : 0.f;
+                if (rc == SOS_OK) gss[b][c] = ms > 0.f ? static_cast<float>(n) * reps / ms / 1e6f : 0.f;
             }
             sos_filter_destroy(f);
         }
         for (int b = 0; b < kTuneBuckets; ++b) {
             int best = 0;
             for (int c = 1; c < kTuneCand; ++c)
-                if (tt.gss[K - 1][b][c] > tt.gss[K - 1][b][best]) best = c;
-            tt.best[K - 1][b] = static_cast<unsigned char>(best);
+                if (gss[b][c] > gss[b][best]) best = c;
+            tt.best[kind][K - 1][b] = static_cast<unsigned char>(best);
         }
     }
     cudaStreamSynchronize(st);
@@ -2273,7 +2290,7 @@ sos_status sos_autotune(int max_log2n, float *report) {
     cudaFree(y);
     if (rc != SOS_OK) return rc;
     tt.valid = true;
-    if (report) std::memcpy(report, tt.gss, sizeof tt.gss);
+    if (report) std::memcpy(report, tt.gss[0], sizeof tt.gss[0]);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune[device] = tt;
     return SOS_OK;
@@ -2284,7 +2301,7 @@ sos_status sos_autotune_choice_ex(int n_sections, int64_t n, int *solver, int *N
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) return SOS_ECUDA;
     int W = 0;
-    if (!tuned_choice(device, n_sections, n, solver, N, &W)) {
+    if (!tuned_choice(device, n_sections, n, true, solver, N, &W)) {
         *solver = 0;
         *N = 0;
         W = 0;

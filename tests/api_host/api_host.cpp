@@ -33,10 +33,12 @@ struct Launch {
     int kind, K, N, norm;
     long long grid;
     std::vector<unsigned char> params;
+    bool strips = false;  // the strip kernel would run
 };
 std::vector<Launch> g_launches;
 bool g_light = false;          // record no parameter blocks and skip the marker (timing runs)
 float g_cost[7][3][9] = {};    // simulated time of a launch, ms, by kind, N (32, 64, 128) and K
+float g_strip_cost[9] = {};    // that of a launch by strips, by K (0: as any other)
 
 int n_index(int N) { return N == 32 ? 0 : N == 64 ? 1 : 2; }
 
@@ -48,7 +50,7 @@ void record(int kind, int K, int N, bool norm, long long grid, const P &p) {
     struct Done {
         ~Done() { g_recording = false; }
     } done;
-    Launch l{kind, K, N, norm ? 1 : 0, grid, {}};
+    Launch l{kind, K, N, norm ? 1 : 0, grid, {}, false};
     if (!g_light) {
         l.params.resize(sizeof(P));
         std::memcpy(l.params.data(), &p, sizeof(P));
@@ -141,7 +143,7 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b) {
     double t = 0.0;
     for (size_t i = a->mark; i < b->mark && i < g_launches.size(); ++i) {
         const Launch &l = g_launches[i];
-        const float c = g_cost[l.kind][n_index(l.N)][l.K];
+        const float c = l.strips && g_strip_cost[l.K] > 0.f ? g_strip_cost[l.K] : g_cost[l.kind][n_index(l.N)][l.K];
         t += c > 0.f ? c : 1.0;
     }
     *ms = static_cast<float>(t);
@@ -179,6 +181,7 @@ cudaError_t launch_dccr(int K, int N, bool norm, int, const PassParams &p, long 
     template <>                                                                                        \
     cudaError_t launch_lane<K, N, W>(bool norm, const LaneParams<K> &p, long long grid, cudaStream_t) {  \
         record(1, K, N, norm, grid, p);                                                                \
+        g_launches.back().strips = p.cut.n_strips > 0;                                                 \
         mark(p.x, p.y, p.n, p.zi, p.zf, K);                                                            \
         return cudaSuccess;                                                                            \
     }
@@ -225,6 +228,7 @@ cudaError_t launch_batch_all(const BatchAllParams &p, long long grid, cudaStream
                              cudaStream_t) {                                                                 \
         if (!img || !gtail) return cudaErrorInvalidValue;                                                    \
         record(6, K, 64, false, grid, p);                                                                    \
+        g_launches.back().strips = p.cut.n_strips > 0;                                                       \
         mark(p.x, p.y, p.n, p.zi, p.zf, K);                                                                  \
         return cudaSuccess;                                                                                  \
     }
@@ -275,6 +279,7 @@ int host_run_scratch(sos_filter *f, const float *x, float *y, long long n, const
     return rc;
 }
 void host_reset(void) { g_launches.clear(); }
+void host_set_strip_cost(int K, float ms) { g_strip_cost[K] = ms; }
 void host_set_light(int on) { g_light = on != 0; }
 void host_set_capturing(int on) { g_capturing = on != 0; }
 void host_set_cost(int kind, int N, int K, float ms) { g_cost[kind][n_index(N)][K] = ms; }

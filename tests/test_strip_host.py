@@ -2,13 +2,14 @@
 stand-ins of tests/api_host/): the rows after which a state is forgotten, the cascade's float32 noise, and the rule
 that cuts a signal into strips (sosfilt_strip_rule.h)."""
 import ctypes
+import shutil
 
 import numpy as np
 import pytest
 
 from workloads import designs
 
-from .test_api_host import _create, lib  # noqa: F401  (a fixture)
+from .test_api_host import _LIB, KIND_LANE, KIND_TC, _create, _launches, _tune_costs, lib  # noqa: F401  (a fixture)
 
 ROW = 64
 SMS = 152  # of the device on which the rule's lines were measured; the stand-in has four
@@ -195,3 +196,45 @@ def _settled_noise(sos):
             z[i] = Z
         v, w = y, z
     return float(np.linalg.norm(v[skip:] - w[skip:]) / np.linalg.norm(w[skip:]))
+
+
+def test_the_autotuner_keeps_a_choice_for_runs_by_strips_and_one_for_the_others(lib, tmp_path):  # noqa: F811
+    """Where strips make the PH solver as fast as the tensor-core one, the choice for runs that keep the lookback
+    is still the tensor cores'.  On a copy of the library, whose tuning no other test sees."""
+    shared, path = lib, tmp_path / "libapi_host.so"
+    shutil.copy(_LIB, path)
+    lib = ctypes.CDLL(str(path))
+    for name in ("sos_filter_create", "sos_filter_destroy", "sos_filter_run", "host_launch"):
+        getattr(lib, name).argtypes = getattr(shared, name).argtypes
+        getattr(lib, name).restype = getattr(shared, name).restype
+    lib.sos_autotune.argtypes = [ctypes.c_int, ctypes.c_void_p]
+    lib.host_set_strip_cost.argtypes = [ctypes.c_int, ctypes.c_float]
+    lib.host_set_cost.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_float]
+    K, n = 8, 1 << 20
+
+    def kinds(sos, n=n, offset=0):
+        f = _create(lib, sos)
+        x = np.zeros(n + 8, np.float32)
+        at = x.ctypes.data + (-x.ctypes.data) % 16 + 4 * offset
+        lib.host_reset()
+        assert lib.sos_filter_run(f, at, at, n, None, None, None) == 0
+        got = [(l["kind"], l["N"]) for l in _launches(lib)]
+        lib.sos_filter_destroy(f)
+        return got
+
+    def tune():
+        lib.host_set_light(1)
+        try:
+            assert lib.sos_autotune(20, None) == 0
+        finally:
+            lib.host_set_light(0)
+            lib.host_reset()
+
+    _tune_costs(lib, lambda K: (KIND_TC, 64))       # lookback: the tensor cores are the fastest
+    for k in range(1, 9):
+        lib.host_set_strip_cost(k, 0.5)             # strips: both solvers are equal, the first is kept
+    tune()
+    assert kinds(designs.butter_lowpass(2 * K, 0.2)) == [(KIND_LANE, 64)]
+    assert kinds(_resonator(K, 0.999)) == [(KIND_TC, 64)]                   # too noisy
+    assert kinds(_resonator(K, 0.99999)) == [(KIND_TC, 64)]                 # remembers too long
+    assert kinds(designs.butter_lowpass(2 * K, 0.2), n=60000) == [(KIND_TC, 64)]  # too short
