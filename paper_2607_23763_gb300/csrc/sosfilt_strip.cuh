@@ -441,24 +441,92 @@ __device__ __forceinline__ void put4(float *y, int k, int from, int to, const fl
     }
 }
 
-// The `count` samples of the row at sample `at`, by the sections one after the other from the row's state
-// (transposed direct form II), from the signal to the output directly.  For rows whose products are worth
-// nothing: rare, and small rather than fast.
+// A warp's rows whose products are worth nothing (`bad`), from the signal to the output directly: by the sections one
+// after the other (transposed direct form II) from the rows' states, which are in the 16 + 16 columns at d.  The group's
+// first sample is `base`, its own are from .. to - 1.  Rare, and small rather than fast.
 template <int K>
-__device__ __noinline__ void row_plainly(const LaneParams<K> &p, long long at, int count, const float (&st)[16]) {
-    float z[2 * K];
-    for (int s = 0; s < 2 * K; ++s) z[s] = st[s];
-    for (int m = 0; m < count; ++m) {
-        float v = p.x[at + m] * p.gain;
-        for (int s = 0; s < K; ++s) {
-            const float4 c = p.sec[s].c;  // b1, b2, -a1, -a2
-            const float y = fmaf(p.sec[s].b0, v, z[2 * s]);
-            z[2 * s] = fmaf(c.x, v, fmaf(c.z, y, z[2 * s + 1]));
-            z[2 * s + 1] = fmaf(c.y, v, c.w * y);
-            v = y;
+__device__ __noinline__ void rows_plainly(const LaneParams<K> &p, unsigned d, bool bad, long long base, int from, int to) {
+    float e[16], l[16];
+    tc_ldn<16>(d, e);
+    tc_ldn<16>(d + 16, l);
+    tc_wait_ld();
+    const int k = (threadIdx.x & 31) * kStripN;
+    if (bad && k >= from && k < to) {
+        const long long at = base + k;
+        const int count = to - k < kStripN ? to - k : kStripN;
+        float z[2 * K];
+        for (int s = 0; s < 2 * K; ++s) z[s] = e[s] + l[s];
+        for (int m = 0; m < count; ++m) {
+            float v = p.x[at + m] * p.gain;
+            for (int s = 0; s < K; ++s) {
+                const float4 c = p.sec[s].c;  // b1, b2, -a1, -a2
+                const float y = fmaf(p.sec[s].b0, v, z[2 * s]);
+                z[2 * s] = fmaf(c.x, v, fmaf(c.z, y, z[2 * s + 1]));
+                z[2 * s + 1] = fmaf(c.y, v, c.w * y);
+                v = y;
+            }
+            p.y[at + m] = v;
         }
-        p.y[at + m] = v;
     }
+    __syncwarp();
+}
+
+// In place: a strip's warm-up samples have been read.  (Out of line, as rows_again: code that hardly ever runs costs the
+// epilogue's loop a few per cent by its layout alone.)
+static __device__ __noinline__ void set_flag(unsigned *flag, bool now) {
+    if (!now) return;
+    __threadfence();
+    atomicExch(flag, 1u);
+}
+
+// The terminal states of a warp's rows (R the first of them), in the accumulator d, again: where they are not finite
+// (`bad`), which samples next to the largest float32 bring about as well as ones that are not finite, from the samples by
+// FMAs -- with outputs from the signal, up to the strip's end, since the stage is gone; otherwise from the row X of it.
+template <int K, int MODE>
+__device__ __noinline__ void rows_again(const LaneParams<K> &p, unsigned d, bool bad, long long R, long long r_end,
+                                        const unsigned char *X) {
+    const long long at = (R + (threadIdx.x & 31)) * kStripN, end = r_end * kStripN < p.n ? r_end * kStripN : p.n;
+    constexpr int S = 2 * K;
+    constexpr bool MM = MODE == kStripOutputs;
+    float t[16], a[16];
+    tc_ldn<16>(d + (MM ? 64 : 0), t);
+    tc_wait_ld();
+    if constexpr (!MM) {  // as the epilogue adds them
+        float b[16];
+        tc_ldn<16>(d + 32, a);
+        tc_wait_ld();
+        for (int j = 0; j < 16; ++j) t[j] += a[j];
+        tc_ldn<16>(d + 16, a);
+        tc_ldn<16>(d + 48, b);
+        tc_wait_ld();
+        for (int j = 0; j < 16; ++j) t[j] += a[j] + b[j];
+    }
+    if (bad) {
+        const int r = static_cast<int>(reinterpret_cast<uintptr_t>(X) >> 7) & 7;
+        for (int s = 0; s < S; ++s) {
+            float v = 0.f;
+            for (int j = 0; j < kStripN; ++j) {
+                float x = 0.f;
+                if constexpr (MM) {
+                    if (at + j < end) x = p.x[at + j];
+                } else {
+                    const int c = j & 31;
+                    x = *reinterpret_cast<const float *>(X + (j >> 5) * kStripHalf + ((((c >> 2) ^ r) << 4) | ((c & 3) << 2)));
+                }
+                v = fmaf(__ldg(p.gtail + s * kStripN + j), x, v);
+            }
+            t[s] = v;
+        }
+    }
+    __syncwarp();
+    tc_st16(d + (MM ? 64 : 0), t);
+    if constexpr (!MM) {
+        for (int j = 0; j < 16; ++j) a[j] = 0.f;
+        tc_st16(d + 16, a);
+        tc_st16(d + 32, a);
+        tc_st16(d + 48, a);
+    }
+    tc_wait_st();
 }
 
 // Row `row` of y = A x, A dense column-major S x S and x in shared memory (read as pairs, broadcast): no
@@ -806,10 +874,6 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             const unsigned xs = i % XS;
             if (!strip_wait(&full[xs], (i / XS) & 1, budget, p.status)) break;
             if (warp == 4) trace(i, 1);
-            if (P.in_place && warp == 4 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows) {
-                __threadfence();
-                atomicExch(&tail->flag[strip], 1u);  // the warm-up samples have been read
-            }
             const unsigned char *X = sm + xs * kStripXBytes + r * 128;
             bool ok = true;
 #pragma unroll 1
@@ -866,10 +930,6 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             if (ok) {
                 float t[S];
                 if constexpr (!Sd::TC) {
-                    if (P.in_place && q == 0 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows) {
-                        __threadfence();
-                        atomicExch(&tail->flag[strip], 1u);  // the warm-up samples have been read
-                    }
                     const unsigned o = xs * kStripXBytes + r * 128 + ((r & 7) << 4);
                     float a[S][2];
 #pragma unroll
@@ -885,32 +945,42 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     }
 #pragma unroll
                     for (int s = 0; s < S; ++s) t[s] = a[s][0] + a[s][1];
-                } else if constexpr (Sd::MM) {
-                    tc_fence_after();
-                    constexpr int C = S <= 2 ? 2 : S <= 4 ? 4 : S <= 8 ? 8 : 16;
-                    float a[C];
-                    tc_ldn<C>(tl + ds * Sd::COLS + 64, a);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < S; ++j) t[j] = a[j];
-                    bad = !(fabsf(t[0]) <= 3.402823466e38f);
                 } else {
                     tc_fence_after();
                     constexpr int C = S <= 2 ? 2 : S <= 4 ? 4 : S <= 8 ? 8 : 16;
-                    float a0[C], a1[C];
-                    tc_ldn<C>(tl + ds * Sd::COLS + 16, a0);  // the small terms
-                    tc_ldn<C>(tl + ds * Sd::COLS + 48, a1);
-                    tc_wait_ld();
+                    const unsigned d = tl + ds * Sd::COLS;
+                    auto terminal = [&]() {
+                        if constexpr (Sd::MM) {
+                            float a[C];
+                            tc_ldn<C>(d + 64, a);
+                            tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < S; ++j) t[j] = a0[j] + a1[j];
-                    tc_ldn<C>(tl + ds * Sd::COLS, a0);
-                    tc_ldn<C>(tl + ds * Sd::COLS + 32, a1);
-                    tc_wait_ld();
+                            for (int j = 0; j < S; ++j) t[j] = a[j];
+                        } else {
+                            float a0[C], a1[C];
+                            tc_ldn<C>(d + 16, a0);  // the small terms
+                            tc_ldn<C>(d + 48, a1);
+                            tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < S; ++j) t[j] = (a0[j] + a1[j]) + t[j];
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&dfree[ds]);
+                            for (int j = 0; j < S; ++j) t[j] = a0[j] + a1[j];
+                            tc_ldn<C>(d, a0);
+                            tc_ldn<C>(d + 32, a1);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int j = 0; j < S; ++j) t[j] = (a0[j] + a1[j]) + t[j];
+                        }
+                    };
+                    terminal();
+                    bad = !(fabsf(t[0]) <= 3.402823466e38f);
+                    if (__any_sync(0xffffffffu, bad)) {
+                        rows_again<K, MODE>(p, d, bad, R, r_end, sm + xs * kStripXBytes + r * 128);
+                        terminal();
+                    }
+                    if constexpr (!Sd::MM) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&dfree[ds]);
+                    }
                 }
                 if (q == 0) trace(i, 5);
                 if constexpr (Sd::MM) scan2<K>(p, cs, t, Sl, ab + q * S, lane);
@@ -936,6 +1006,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             if (!Sd::MM && dead) continue;
             if (q == 0) trace(i, 9);
             const float *z0 = z_buf + (i % kStripZ) * S;
+            // the unit's rows have all been read, and the ones before, by rows_again too
+            if (P.in_place) set_flag(&tail->flag[strip], q == 0 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows);
             if (q == QC) {
                 const float zn = (HALVES ? mv_two<S>(A4, z0, A1, ab + 2 * S, lane) : mv_shared<S>(A4, z0, li)) + cu;
                 if (i + 1 < n_u) {
@@ -1121,14 +1193,7 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
                     if (bad_rows && !dead) {
                         // rows with samples that are not finite: the outputs up to the first of them are right
                         // by the recurrence, which is run from the rows' states on the signal itself
-                        float e[16], l[16];
-                        tc_ldn<16>(tl + ds * Sd::COLS + 64, e);
-                        tc_ldn<16>(tl + ds * Sd::COLS + 80, l);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) e[j] += l[j];
-                        const int k = lane * kStripN;
-                        if (bad && k >= from && k < to) row_plainly<K>(p, base + k, to - k < kStripN ? to - k : kStripN, e);
+                        rows_plainly<K>(p, tl + ds * Sd::COLS + 64, bad, base, from, to);
                         __syncwarp();
                     }
                     if (!dead) {

@@ -303,3 +303,27 @@ def test_both_ways_agree_where_the_rule_changes(dev, order, cutoff, n):
             assert float((za - zb).abs().max()) < 2e-5 * float(zb.abs().max())
         a.close()
     b.close()
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("long", [False, True])
+@pytest.mark.parametrize("order,cutoff,solver", [(2, 0.2, 0), (4, 0.3, 0), (8, 0.5, 0), (6, 0.5, 0), (16, 0.05, 0), (8, 0.1, 4)])
+def test_samples_next_to_the_largest_float32(dev, order, cutoff, solver, long, in_place):
+    """Finite outputs where the lookback kernel's are, though such samples round to an infinite TF32 value; in own
+    rows and in the rows that warm the next strip up."""
+    sos = designs.butter_lowpass(order, cutoff)
+    n = _long(dev, order) + 77 if long else (1 << 20) + 77
+    x = 1e36 * torch.randn(n, device=dev, generator=torch.Generator(device=dev).manual_seed(order))
+    x[5] = -3.4028234e38
+    x[20011::50021] = 3.4028234e38
+    x[-3] = 3.4028e38
+    f, g = _filter(sos, tuning={"solver": solver}), _filter(sos, tuning={"solver": 2, "groups_per_cta": 10})
+    zf, zg = torch.empty(order // 2, 2, device=dev), torch.empty(order // 2, 2, device=dev)
+    want = g.run(x, zf=zg)
+    y = f.run(x, x if in_place else None, zf=zf)
+    assert f.sync_status() == 0 and g.sync_status() == 0
+    assert bool(torch.isfinite(want).all()) and bool(torch.isfinite(zg).all())
+    assert float((y - want).abs().max()) < 2e-5 * float(want.abs().max())
+    assert float((zf - zg).abs().max()) < 2e-5 * float(zg.abs().max())
+    f.close()
+    g.close()
