@@ -284,6 +284,7 @@ def run_batch(filters, xs, ys=None, zis=None, zfs=None, stream=None):
     n = len(xs)
     if ys is None:
         ys = [torch.empty_like(x) for x in xs]
+    ys = ys if isinstance(ys, (list, tuple)) else list(ys)
     filters = filters if isinstance(filters, (list, tuple)) else list(filters)
     zis = zis if zis is None or isinstance(zis, (list, tuple)) else list(zis)
     zfs = zfs if zfs is None or isinstance(zfs, (list, tuple)) else list(zfs)
