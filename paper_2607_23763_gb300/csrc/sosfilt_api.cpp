@@ -1338,12 +1338,13 @@ int tune_bucket(int64_t n) {
     return b;
 }
 
-bool tuned_choice(int device, int K, int64_t n, bool strips, int *solver, int *N, int *W) {
+template <class Strips>  // whether the run goes by strips, asked only if there is a choice
+bool tuned_choice(int device, int K, int64_t n, Strips &&strips, int *solver, int *N, int *W) {
     if (device < 0 || device >= 64) return false;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_tune[device].valid) return false;
     const int k = (K > sosk::kMaxPass ? sosk::kMaxPass : K) - 1;
-    candidate(g_tune[device].best[strips ? 0 : 1][k][tune_bucket(n)], solver, N, W);
+    candidate(g_tune[device].best[strips() ? 0 : 1][k][tune_bucket(n)], solver, N, W);
     return true;
 }
 
@@ -1371,7 +1372,7 @@ sos_status run_impl(sos_filter *f, const float *x, float *y, int64_t n, const fl
     if (!t.N && !t.carry && !t.solver && !t.lookback_width && !t.groups_per_cta) {
         // all defaults: the autotuned choice for this section count and length, if there is one
         int solver = 0, N = 0, W = 0;
-        if (tuned_choice(f->device, f->K, n, runs_by_strips(f, x, y, n), &solver, &N, &W)) {
+        if (tuned_choice(f->device, f->K, n, [&] { return runs_by_strips(f, x, y, n); }, &solver, &N, &W)) {
             if (solver == SOS_SOLVER_PH) return run_lane(f, x, y, n, zi, zf, s, N, W);
             if (solver == SOS_SOLVER_DTCR) return run_dtcr(f, x, y, n, zi, zf, s);
             if (solver == SOS_SOLVER_TC) return run_tc(f, x, y, n, zi, zf, s);
@@ -2301,7 +2302,7 @@ sos_status sos_autotune_choice_ex(int n_sections, int64_t n, int *solver, int *N
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) return SOS_ECUDA;
     int W = 0;
-    if (!tuned_choice(device, n_sections, n, true, solver, N, &W)) {
+    if (!tuned_choice(device, n_sections, n, [] { return true; }, solver, N, &W)) {
         *solver = 0;
         *N = 0;
         W = 0;

@@ -930,6 +930,10 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             if (ok) {
                 float t[S];
                 if constexpr (!Sd::TC) {
+                    if (P.in_place && q == 0 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows) {
+                        __threadfence();
+                        atomicExch(&tail->flag[strip], 1u);  // the warm-up samples have been read
+                    }
                     const unsigned o = xs * kStripXBytes + r * 128 + ((r & 7) << 4);
                     float a[S][2];
 #pragma unroll
@@ -1007,7 +1011,8 @@ __global__ void __launch_bounds__(StripDims<K, MODE>::THREADS, 1)
             if (q == 0) trace(i, 9);
             const float *z0 = z_buf + (i % kStripZ) * S;
             // the unit's rows have all been read, and the ones before, by rows_again too
-            if (P.in_place) set_flag(&tail->flag[strip], q == 0 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows);
+            if constexpr (Sd::TC)
+                if (P.in_place) set_flag(&tail->flag[strip], q == 0 && lane == 0 && n_warm > 0 && static_cast<int>(i) == (n_warm - 1) / kStripRows);
             if (q == QC) {
                 const float zn = (HALVES ? mv_two<S>(A4, z0, A1, ab + 2 * S, lane) : mv_shared<S>(A4, z0, li)) + cu;
                 if (i + 1 < n_u) {
