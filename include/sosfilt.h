@@ -27,7 +27,10 @@
  *     the same future outputs: (z1, z2) is exactly the forcing B_ x_-1 - A_ y_-1
  *     on the first two rows of Eq. 2.)
  *   - Samples are float32; arithmetic is float32 (tables are derived in
- *     float64 on the host and rounded once).
+ *     float64 on the host and rounded once).  Runs that use the tensor cores
+ *     (SOS_SOLVER_TC, and runs by strips as described there) take products of
+ *     samples, states and tables split into two TF32 words of 11 bits each,
+ *     accumulated in float32.
  *   - Device pointers are plain CUDA device addresses (e.g. torch tensors'
  *     data_ptr()).  `stream` is a cudaStream_t passed as void* (NULL = the
  *     legacy default stream).  Every call that takes a stream is asynchronous
@@ -93,8 +96,9 @@ enum {
                                float32 operand split into head and remainder (float32 accuracy).
                                Cascade carry only, N = 64, tiles of 8 groups.  Needs x and y
                                16-byte aligned and n >= 64; other runs use SOS_SOLVER_PH.
-                               By strips (below) both solvers use the tensor cores, SOS_SOLVER_PH
-                               for the outputs too where its float32 rounding is no smaller */
+                               By strips (sos_filter_run) both solvers use the tensor cores,
+                               SOS_SOLVER_PH for the outputs too where the cascade's float32
+                               rounding is not below theirs */
 };
 
 /*
@@ -177,6 +181,9 @@ sos_status sos_filter_destroy(sos_filter *f);
  * graph, so every replay starts afresh; it allocates nothing, so the filter must
  * have run once outside the capture on a signal at least as long (else SOS_EINVAL).
  * Replays must not overlap each other or other runs of the same filter.
+ * Which kernel runs (by strips or with lookback) depends on n, on the cascade's
+ * memory and on whether x and y are 16-byte aligned, so that the same samples at
+ * another alignment may come out with other last bits.
  */
 sos_status sos_filter_run(sos_filter *f, const float *x_dev, float *y_dev, int64_t n, const float *zi_dev,
                           float *zf_dev, void *stream);

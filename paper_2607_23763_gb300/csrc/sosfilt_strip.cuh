@@ -1,38 +1,50 @@
 // Persistent single-signal kernel for cascades whose memory is finite in float32, sm_103a: the signal
-// is cut into one strip of consecutive samples per thread block, and no block waits on another.
+// is cut into one strip of consecutive samples per thread block, and no block takes another's state.
 //
 // The zero-input transition of a stable cascade over H samples, M1^H, decays to matrices whose float32
 // entries are all zero; from there on a state H samples old adds nothing to the carried one (Eq. 25 with
 // the terms the float32 tables hold as zeros left out).  The host finds that memory once per filter
 // (warm_rows, in rows of 64 samples).  A block then starts its strip warm_rows rows early from zero state,
 // which gives it the strip's true incoming state, and carries the state from unit to unit inside the
-// block: no lookback across blocks, no descriptors, the same composition on every run.
+// block: no lookback across blocks, no descriptors, the same composition on every run.  Only in place
+// does a block wait for another: a strip's last rows are stored once the next strip has read them as its
+// warm-up (a word per strip; strips are taken from the last one down, so the block waited for is running
+// or done).  Which signals are cut, and how: sosfilt_strip_rule.h.
 //
 // A unit is 128 rows of N = 64 samples, staged in shared memory with the 16-byte chunks of a row permuted
 // by the row number (a lane reads its own row without bank conflicts).  Per unit:
-//   1. terminal states of the rows under zero state (Sec. II-C).  With one or two sections, by FMAs: each
-//      lane multiplies its row with the 2 or 4 state responses.  With more, the product of the rows with the 64
-//      state responses, T = X G^T, by tcgen05.mma with the rows in tensor memory.  TF32 products of the
-//      split operands: X as its upper 19 bits (what the tensor core reads) and the rounded remainder, G
-//      as a TF32 value rounded to nearest and its remainder; the four partial products enter separate
-//      accumulators for the large and the small terms, summed in float32 by the epilogue.
+//   1. terminal states of the rows under zero state (Sec. II-C).
+//      kStripFma (one or two sections, short or misaligned signals): each lane multiplies its row with the
+//      2 or 4 state responses by FMAs.
+//      kStripStates (one or two sections, long; more, quiet): T = X G^T, the rows times the 64 state responses,
+//      by tcgen05.mma with the rows in tensor memory.
+//      kStripOutputs (three sections and more): [Y | T] = X [T^T | G^T], the rows' zero-state outputs by the lower
+//      triangular Toeplitz matrix of the impulse response as well.
+//      The products are of split operands in TF32: the samples as the nearest TF32 values (11 bits) and exact
+//      remainders (12 bits, of which the tensor core reads 11), the tables as nearest TF32 values and remainders
+//      rounded to TF32.  kStripStates takes all four partial products, into separate accumulators for the large and
+//      the small terms, which the epilogue adds; kStripOutputs leaves remainder times remainder out (3 % of the
+//      error) and takes the small terms first, into one accumulator.
 //   2. lane scan (Sec. II-C's recursive doubling) of each warp's 32 rows, fold of the four groups'
 //      carries, and the unit's incoming state Z' = (A_C)^4 Z + c from the previous unit's.
-//   3. every row's true incoming state S_l + (M_N)^l Z (Eq. 24 at the rows' starts), from which the
-//      sections' recurrences run over the row in place, skewed by one sample per section: the outputs
-//      themselves, 4 FMAs per section and sample and no separate correction pass (the lookback kernel's
-//      particular pass and correction are 6).
-//   4. coalesced stores.
-// Groups of warm-up rows stop after step 2.
+//   3. every row's true incoming state S_l + (M_N)^l Z (Eq. 24 at the rows' starts), and from it the outputs:
+//      by the sections' recurrences over the row in place, skewed by one sample per section, 4 FMAs per section
+//      and sample and no separate correction pass (the lookback kernel's particular pass and correction are 6);
+//      or, kStripOutputs, by a second product onto the first, Y += St H^T with the rows' states as an operand of
+//      two TF32 words (three partial products).
+//   4. coalesced stores, through a staging buffer and by TMA where the outputs are in tensor memory.
+// Groups of warm-up rows stop after step 2.  Samples that are not finite, or so large that their nearest TF32
+// value is not: rows_again, rows_plainly; what follows a strip that ends in such a state: the last block.
 //
 // Warp roles (one block per SM; the first eight warps give registers to the others):
-//   warps 0, 2, 3  load the units' samples (cp.async, zero-filled past the end, any alignment)
+//   warps 0, 2, 3  load the units' samples: TMA where x and y are 16-byte aligned and strips long, by one thread;
+//                  else cp.async (zero-filled past the end, any alignment)
 //   warp 1         tensor-memory owner; issues the products
 //   warps 4-7      split the rows into the products' operands, in tensor memory (two buffers)
 //   warps 8 on     three or four warpgroups, one unit each in turn; warp q of a warpgroup takes rows
 //                  32q .. 32q+31
 // Without the tensor cores warps 0-7 all load.
-// Every wait is bounded by the spin budget.
+// Every wait is bounded by the spin budget, and those for a block's own copies and products at its end by kStripDrain.
 #pragma once
 #include <cstring>
 

@@ -27,16 +27,16 @@ struct StripCut {
 struct StripRule {
     // x aligned: the least rows of a signal, with a warm-up of a unit or less and with a longer one.  The general
     // floor of 2048 rows (32 strips of half a unit) is where order 8 breaks even (12.3 us both, recurrences; products
-    // 13.3 at 2^17 samples against 12.3 to 14.3, box by box, 13.3 against 14.3 at 2^18).  Order 6: recurrences 12.3
-    // against 12.4 at 2^18, 10.3 at 2^17; products 13.2 to 14.3 up to 2^20.4 against 12.4 to 13.4, 14.3 against 15.4
-    // at 2^21.  With 200 rows of warm-up (strips of 200 rows and more, so fewer of them): order 8 by products 16.4
-    // against 15.4 at 2^20.6, 16.4 against 16.3 at 2^21.
+    // 13.3 at 2^17 samples against 12.3 to 14.3 from device to device, 13.3 against 14.3 at 2^18).  Order 6:
+    // recurrences 12.3 against 12.4 at 2^18, 10.3 at 2^17; products 13.2 to 14.3 up to 2^20.4 against 12.4 to 13.4,
+    // 14.3 against 15.4 at 2^21.  With 200 rows of warm-up (strips of 200 rows and more, so fewer of them): order 8 by
+    // products 16.4 against 15.4 at 2^20.6, 16.4 against 16.3 at 2^21.
     int least, least_long;
     // x misaligned: least rows; the rows that a strip's units hold, warm-up included, over its own at most; and the
-    // warm-up that signals of less than kStripShortOdd rows may have whatever its share (50 below 4096, except at order 16).  Order 6 by products: 7 units
-    // on 862 rows 32.8 us against 34.0, 8 on 862 36.1, 6 on 611 29 against 26.7.  Order 8 by products: 3 on 305 20.5
-    // against 22.4, 4 on 305 23.8, 5 on 514 27.7 against 27.3.  Order 16: 7 on 432 (0.8 units of it warm-up) 33.1
-    // against 35.5, 18 on 1221 76.1 against 75.4.
+    // warm-up that signals of less than kStripShortOdd rows may have whatever its share (50 below 4096, except at
+    // order 16).  Order 6 by products: 7 units on 862 rows 32.8 us against 34.0, 8 on 862 36.1, 6 on 611 29 against
+    // 26.7.  Order 8 by products: 3 on 305 20.5 against 22.4, 4 on 305 23.8, 5 on 514 27.7 against 27.3.  Order 16: 7 on
+    // 432 (0.8 units of it warm-up) 33.1 against 35.5, 18 on 1221 76.1 against 75.4.
     int least_odd;
     float units_odd;
     int warm_odd;
@@ -53,9 +53,9 @@ inline const StripRule &strip_rule(int K, bool products) {
     return (products ? prod : rec)[K - 3];
 }
 
-// One or two sections: a strip no longer than this many rows and its warm-up's (1600 at most), and any where x is misaligned,
-// takes its terminal states by FMAs (no operands, products or tensor memory on the way, and eight warps load).  Longer
-// ones on the tensor cores, with TMA.  Order 2: 2^24.5 samples 38.0 us against 40.5, 2^25 51.6 against 50.7 (with 1600
+// One or two sections: a strip no longer than this many rows and its warm-up's (1600 at most), and any where x is
+// misaligned, takes its terminal states by FMAs (no operands, products or tensor memory on the way, and eight warps
+// load).  Longer ones on the tensor cores, with TMA.  Order 2: 2^24.5 samples 38.0 us against 40.5, 2^25 51.6 against 50.7 (with 1600
 // rows of warm-up 55.5 against 57.9), 2^28 352 against 333; order 4: 2^26 93.5 against 99.1, 2^27 183 against 181.
 // Misaligned, 2^28: order 2 431 against 545 (lookback 572), order 4 455 against 593 (636).
 inline int strip_fma_rows(int K) { return K == 1 ? 3328 : 12288; }
@@ -104,9 +104,10 @@ inline bool strip_cut(int K, bool products, bool odd, bool tc, long long n, int 
             const long long units = (per + warm_rows + kStripRows - 1) / kStripRows;
             const int any = c.n_rows >= kStripShortOdd ? 0 : c.n_rows < 4096 && K < 8 && r.warm_odd > 50 ? 50 : r.warm_odd;
             if (warm_rows > any && units * kStripRows > r.units_odd * strip) return false;
-        } else if (warm_rows > (per > 2 * kStripRows ? per : 2 * kStripRows) || (tc && K <= 4 && per > 1024 && warm_rows > 0.7 * strip)) {
-            // three and four sections against the tensor-core lookback kernel: even at 0.9 of a strip (2^28, order 6: 457 us
-            // against 486 at 0.7, 507 against 484 at 1); the others win with a warm-up as long as the strip
+        } else if (warm_rows > (per > 2 * kStripRows ? per : 2 * kStripRows) ||
+                   (tc && K <= 4 && per > 1024 && warm_rows > 0.7 * strip)) {
+            // three and four sections against the tensor-core lookback kernel: even at 0.9 of a strip (2^28, order 6:
+            // 457 us against 486 at 0.7, 507 against 484 at 1); the others win with a warm-up as long as the strip
             return false;
         }
     }

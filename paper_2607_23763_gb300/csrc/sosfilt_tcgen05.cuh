@@ -37,16 +37,7 @@ __device__ __forceinline__ unsigned tc_elect() {
 
 // Products issued by a whole warp, the elected lane's (`go`) being carried out: in converged code the
 // operands are uniform registers, and a product costs what the tensor core takes (128 rows, K = 8: N / 2
-// cycles with A in tensor memory, 36 + N / 4 with A in shared memory).  Issued from a branch of one lane
-// the operands' moves take 45 cycles each.
-__device__ __forceinline__ void tc_mma_ss(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc,
-                                          unsigned acc, unsigned go) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(go)
-        : "memory");
-}
+// cycles with A in tensor memory).  Issued from a branch of one lane the operands' moves take 45 cycles each.
 // A in tensor memory (lanes: rows, 8 columns of 32 bits per product).
 __device__ __forceinline__ void tc_mma_ts(unsigned d, unsigned a, unsigned long long b, unsigned idesc, unsigned acc,
                                           unsigned go) {
